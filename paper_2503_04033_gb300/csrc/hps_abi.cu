@@ -228,7 +228,7 @@ void lu_factor(const Plan& P, Work<T>& w, int nbox, int* status, cudaStream_t st
             a.B = w.G; a.ldb = ldm; a.sB = w.sG;
             a.O = w.M + (long long)k * ldm + c0; a.ldo = ldm; a.sO = w.sM;
             a.M = n - k; a.N = nc; a.K = nb; a.mode = GM_FWD; a.split = nb;
-            a.perm = Ps; a.sP = w.sP; a.W = w.W; a.ldw = ldm; a.sW = w.sG;
+            a.perm = Ps; a.sP = w.sP; a.W = w.W; a.ldw = ldm; a.sW = w.sG; a.status = status;
             launch_gemm<T>(a, nbox, st);
         }
     }

@@ -20,7 +20,8 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 enum RhsKind { RHS_DTN = 0, RHS_LOAD = 1, RHS_TRACE = 2, RHS_DTN_LOAD = 3 };
 
 // Update-product epilogue modes (see gemm description in hps_kernels.cuh).
-enum GemmMode { GM_SET = 0, GM_ACC = 1, GM_FWD = 2, GM_BWD = 3 };
+// GM_SRC (digit products only): src is row r of W.
+enum GemmMode { GM_SET = 0, GM_ACC = 1, GM_FWD = 2, GM_BWD = 3, GM_SRC = 4 };
 
 // Per-(p, h) device tables: physical first and second derivative matrices,
 // [3][p][p] each (axis-major), FP64.
@@ -107,6 +108,7 @@ struct GemmArgs {
     const int* perm; long long sP;   // GM_FWD: source row of local row r (relative)
     const T* W; long long ldw, sW;   // GM_FWD: saved rows of the panel
     const int* skip;                 // per box: nonzero = leave untouched
+    int* status;                     // per box: HPS_ETIMEOUT when a bounded wait gave up (may be NULL)
 };
 
 // ---------------------------------------------------------------- LU plans
@@ -297,6 +299,10 @@ void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c
 
 template <typename T>
 void launch_gemm(const GemmArgs<T>& a, int nbox, cudaStream_t st);
+
+// FP64 product on the tensor cores from exact 8-bit digits (hps_digit.cu): any
+// M, N, K and mode, B optionally given transposed ([n][k], k contiguous).
+void launch_digit_gemm(const GemmArgs<double>& a, bool b_transposed, int nbox, cudaStream_t st);
 
 void launch_dn(const Geometry& g, int nbox, const double* X, long long ldx, long long sX,
                int ncols, double* out, long long sOut, int transposed_out, int add_abb,
