@@ -202,7 +202,7 @@ void lu_factor(const Plan& P, Work<T>& w, int nbox, int* status, cudaStream_t st
         T* Fs = w.F + P.fw_off[s];
         T* Bs = w.B + P.bw_off[s];
         int* Ps = w.perm + P.perm_off[s];
-        launch_panel<T>(w.M, ldm, w.sM, n, k, nb, P.ib, Ps, w.sP, Fs, NB, w.sF, Bs + (long long)k * NB, NB, w.sB,
+        launch_panel<T>(w.M, ldm, w.sM, n, k, nb, Ps, w.sP, Fs, NB, w.sF, Bs + (long long)k * NB, NB, w.sB,
                         status, nullptr, nbox, st);
         if (n - k - nb > 0) {
             GemmArgs<T> a = gargs<T>();

@@ -80,7 +80,7 @@ struct IfLevel {
     double* y = nullptr;      // solve: W^{-1} (h^a_3 + h^b_3) [nn][s_pad][nrhs]
 };
 
-constexpr int kMaxSeparator = 14000;   // the panel keeps a column of W in shared memory
+constexpr int kMaxSeparator = 14000;   // a panel's cluster holds 16,384 rows
 constexpr int kRefineMax = 10;         // FP32_IR: most corrections per solve
 constexpr double kRefineTol = 1e-14;   // FP32_IR: stop when ||du|| <= tol ||u||
 

@@ -13,7 +13,6 @@ namespace hps {
 
 constexpr int kMaxP = 24;
 constexpr int kMaxNB = 128;          // largest LU block (K of every update product)
-constexpr int kPanelThreads = 512;   // threads of the panel-factorisation CTA
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -114,7 +113,7 @@ struct GemmArgs {
 // ---------------------------------------------------------------- LU plans
 
 struct Plan {
-    int n = 0, r = 0, NB = 0, ib = 0, nsteps = 0;
+    int n = 0, r = 0, NB = 0, nsteps = 0;
     long long ldm = 0;
     size_t elt = 0;                  // bytes per LU element
     bool tc = false;                 // FP32 products on the tensor cores
@@ -152,13 +151,6 @@ inline Plan make_plan(int n, int r, hps_precision prec, int nb_opt, bool use_tc,
     if (NB > kMaxNB) NB = kMaxNB;
     P.NB = NB;
     P.ldm = (long long)align_up((size_t)(n + r), 8);
-    // panel inner-block width: the block column of the panel lives in shared memory
-    const size_t static_smem = 32 * kMaxNB * P.elt + 2048;
-    const size_t budget = 227 * 1024 - static_smem;
-    int ib = 32;
-    while (ib > 1 && (size_t)ib * n * P.elt + (size_t)n * 5 > budget) ib >>= 1;
-    if (ib > NB) ib = NB;
-    P.ib = ib;
     for (int k = 0; k < n; k += NB) {
         const int nb = std::min(NB, n - k);
         P.k0.push_back(k);
@@ -287,9 +279,8 @@ void launch_build_aug(const Geometry& g, double kappa, const double* kappa_box, 
                       const double* beta = nullptr);
 
 template <typename T>
-void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int ib,
-                  int* perm, long long sP, T* Ftop, long long ldf, long long sF,
-                  T* Btop, long long ldb, long long sB, int* status, const int* skip,
+void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* perm, long long sP, T* Ftop,
+                  long long ldf, long long sF, T* Btop, long long ldb, long long sB, int* status, const int* skip,
                   int nbox, cudaStream_t st);
 
 template <typename T>

@@ -1,7 +1,7 @@
 // CUDA-core kernels of the leaf reduction: operator assembly, the blocked LU
-// with partial pivoting (panel factorisation with warp-shuffle pivot search),
-// the row-gather and update products that carry the triangular solves, the
-// FP64 refinement residual, and the D_n / flux products.
+// with partial pivoting (its panels are in hps_panel.cu), the row-gather and
+// update products that carry the triangular solves, the FP64 refinement
+// residual, and the D_n / flux products.
 //
 // Storage of one box's working matrix M (row-major, leading dimension ldm):
 //   M = [ A_ii | RHS ]   n rows, n + r used columns,
@@ -37,9 +37,6 @@ namespace hps {
 namespace {
 
 __device__ __forceinline__ int imin(int a, int b) { return a < b ? a : b; }
-
-template <typename T>
-__device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
 
 // Conversions between FP64 and FP32 on the integer pipe (on GB300 the FP64
 // pipe that executes the conversion instructions is the residual's and the
@@ -286,339 +283,6 @@ __global__ void k_apply_op(int p, int nfield, const double* __restrict__ D2, dou
             }
         }
         ob[idx] = -acc + conv - kappa2 * __ldg(b + box * sb + idx) * us[idx];
-    }
-}
-
-// ---------------------------------------------------------------- panel
-
-// Arg-max of |value| over the CTA with ties to the lowest index.
-template <typename T>
-__device__ __forceinline__ void argmax_merge(T& v, int& i, T ov, int oi)
-{
-    if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
-}
-
-// Inverse of a triangle held in A (P x P, row-major, P a power of two >= 16,
-// padded with the identity): the unit lower triangle below A's diagonal
-// (lower) or the upper triangle with its diagonal.  The 16 x 16 diagonal
-// blocks are inverted by substitution (a column per thread), then blocks of
-// doubling size b are joined: for [[A1, 0], [C, D]] the off-diagonal block
-// of the inverse is -D^{-1} (C A1^{-1}); for [[A1, B], [0, D]] it is
-// -A1^{-1} (B D^{-1}).  The middle product is parked in the free triangle of
-// A.  X must be zero on entry and receives the inverse.  A zero diagonal
-// entry is read as 1 (the box is already flagged singular).
-template <typename T>
-__device__ void tri_inverse(T* A, T* X, int P, bool lower, int tid)
-{
-    if (tid < P) {
-        const int q0 = (tid >> 4) << 4, c = tid;
-        if (lower) {
-            X[c * P + c] = T(1);
-            for (int r = c + 1; r < q0 + 16; ++r) {
-                T acc = T(0);
-                for (int t = c; t < r; ++t) acc -= A[r * P + t] * X[t * P + c];
-                X[r * P + c] = acc;
-            }
-        } else {
-            T d = A[c * P + c];
-            if (d == T(0)) d = T(1);
-            X[c * P + c] = T(1) / d;
-            for (int r = c - 1; r >= q0; --r) {
-                T acc = T(0);
-                for (int t = r + 1; t <= c; ++t) acc -= A[r * P + t] * X[t * P + c];
-                T dr = A[r * P + r];
-                if (dr == T(0)) dr = T(1);
-                X[r * P + c] = acc / dr;
-            }
-        }
-    }
-    __syncthreads();
-    for (int b = 16; b < P; b *= 2) {
-        const int items = (P / (2 * b)) * b * b;
-        // middle products into the free triangle of A
-        for (int it = tid; it < items; it += kPanelThreads) {
-            const int pr = it / (b * b), e = it - pr * b * b, r = e / b, c = e - r * b, i0 = 2 * b * pr;
-            T acc = T(0);
-            if (lower) {   // C A1^{-1}: C = A[i0+b+r][i0+t], A1^{-1} lower
-                for (int t = c; t < b; ++t) acc += A[(i0 + b + r) * P + i0 + t] * X[(i0 + t) * P + i0 + c];
-                A[(i0 + r) * P + i0 + b + c] = acc;
-            } else {       // B D^{-1}: B = A[i0+r][i0+b+t], D^{-1} upper
-                for (int t = 0; t <= c; ++t) acc += A[(i0 + r) * P + i0 + b + t] * X[(i0 + b + t) * P + i0 + b + c];
-                A[(i0 + b + r) * P + i0 + c] = acc;
-            }
-        }
-        __syncthreads();
-        for (int it = tid; it < items; it += kPanelThreads) {
-            const int pr = it / (b * b), e = it - pr * b * b, r = e / b, c = e - r * b, i0 = 2 * b * pr;
-            T acc = T(0);
-            if (lower) {   // -D^{-1} (C A1^{-1}), D^{-1} lower
-                for (int t = 0; t <= r; ++t) acc -= X[(i0 + b + r) * P + i0 + b + t] * A[(i0 + t) * P + i0 + b + c];
-                X[(i0 + b + r) * P + i0 + c] = acc;
-            } else {       // -A1^{-1} (B D^{-1}), A1^{-1} upper
-                for (int t = r; t < b; ++t) acc -= X[(i0 + r) * P + i0 + t] * A[(i0 + b + t) * P + i0 + c];
-                X[(i0 + r) * P + i0 + b + c] = acc;
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// One CTA factors one box's panel M[k:n, k:k+nb] (Algorithm 1's batched LU,
-// P A_ii = L U with partial pivoting).  The panel is processed in inner blocks
-// of ib columns that live in shared memory (column-major, R rows, in the order
-// the rows were loaded; pos2row maps a pivot position to its loaded row); the
-// pivot search is a warp-shuffle arg-max followed by a cross-warp pass.  After the
-// panel: the step's row permutation perm[r] (source row of local row r),
-// F top = -L11^{-1} and B top = -U11^{-1}.
-constexpr int kSwapPer = (64 * kMaxNB + kPanelThreads - 1) / kPanelThreads;
-
-template <typename T>
-__global__ void __launch_bounds__(kPanelThreads)
-k_panel(T* __restrict__ M, long long ldm, long long sM, int n, int k, int nb, int ib,
-        int* __restrict__ perm, long long sP, T* __restrict__ Ftop, long long ldf, long long sF,
-        T* __restrict__ Btop, long long ldb, long long sB, int* status, const int* skip)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* Sb = reinterpret_cast<T*>(smem_raw);
-    const int R0 = n - k;
-    unsigned short* pos2row = reinterpret_cast<unsigned short*>(smem_raw + (size_t)ib * R0 * sizeof(T));
-    unsigned short* row2pos = pos2row + R0;
-    unsigned char* active = reinterpret_cast<unsigned char*>(row2pos + R0);
-    __shared__ int swp[kMaxNB];
-    __shared__ T red_v[2][kPanelThreads / 32];
-    __shared__ int red_i[2][kPanelThreads / 32];
-    __shared__ int s_sing, s_nmv;
-    __shared__ unsigned short mv[64];
-    __shared__ T Xs[32 * kMaxNB];
-
-    const int box = blockIdx.x;
-    if (skip && skip[box]) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = kPanelThreads / 32;
-    T* Mb = M + box * sM;
-    if (tid == 0) s_sing = 0;
-
-    for (int jb = 0; jb < nb; jb += ib) {
-        const int w = imin(ib, nb - jb);
-        const int R = R0 - jb;
-        T* base = Mb + (long long)(k + jb) * ldm + (k + jb);
-        for (int idx = tid; idx < R * w; idx += kPanelThreads) {
-            const int r = idx / w, c = idx - r * w;
-            Sb[c * R + r] = base[(long long)r * ldm + c];
-        }
-        for (int r = tid; r < R; r += kPanelThreads) {
-            pos2row[r] = (unsigned short)r;
-            row2pos[r] = (unsigned short)r;
-            active[r] = 1;
-        }
-        __syncthreads();
-        // Rows stay where they were loaded; interchanges are tracked in
-        // pos2row/row2pos and applied when the block is written back.  Each
-        // thread owns rows tid, tid + 512, ...; the arg-max candidates of the
-        // next column are formed during this column's update, so every pivot
-        // column costs one barrier.  Ties go to the lowest loaded row.
-        {
-            T bv = T(-1);
-            int bi = INT_MAX;
-            for (int r = tid; r < R; r += kPanelThreads) argmax_merge(bv, bi, tabs(Sb[r]), r);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const T ov = __shfl_xor_sync(0xffffffffu, bv, off);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-                argmax_merge(bv, bi, ov, oi);
-            }
-            if (lane == 0) { red_v[0][warp] = bv; red_i[0][warp] = bi; }
-        }
-        __syncthreads();
-        for (int c = 0; c < w; ++c) {
-            const int cur = c & 1;
-            T bv = red_v[cur][0];
-            int bi = red_i[cur][0];
-#pragma unroll
-            for (int q = 1; q < NW; ++q) argmax_merge(bv, bi, red_v[cur][q], red_i[cur][q]);
-            // Candidates come from rows still active, so a valid index needs no
-            // further test; none (every |value| NaN) keeps the row in place.
-            int pr = bi;
-            if (pr < 0 || pr >= R) pr = pos2row[c];
-            if (tid == 0) {
-                const int pp = row2pos[pr], qr = pos2row[c];
-                pos2row[c] = (unsigned short)pr;
-                pos2row[pp] = (unsigned short)qr;
-                row2pos[pr] = (unsigned short)c;
-                row2pos[qr] = (unsigned short)pp;
-                swp[jb + c] = jb + pp;
-                active[pr] = 0;
-            }
-            T piv = Sb[c * R + pr];
-            if (piv == T(0)) {
-                // Exactly singular: record it and keep the arithmetic finite.
-                if (tid == 0) s_sing = 1;
-                piv = T(1);
-            }
-            const T rinv = T(1) / piv;
-            T nv = T(-1);
-            int ni = INT_MAX;
-            for (int r = tid; r < R; r += kPanelThreads) {
-                if (r == pr || !active[r]) continue;
-                const T l = Sb[c * R + r] * rinv;
-                Sb[c * R + r] = l;
-                for (int cc = c + 1; cc < w; ++cc) Sb[cc * R + r] -= l * Sb[cc * R + pr];
-                if (c + 1 < w) argmax_merge(nv, ni, tabs(Sb[(c + 1) * R + r]), r);
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const T ov = __shfl_xor_sync(0xffffffffu, nv, off);
-                const int oi = __shfl_xor_sync(0xffffffffu, ni, off);
-                argmax_merge(nv, ni, ov, oi);
-            }
-            if (lane == 0) { red_v[cur ^ 1][warp] = nv; red_i[cur ^ 1][warp] = ni; }
-            __syncthreads();
-        }
-        for (int idx = tid; idx < R * w; idx += kPanelThreads) {
-            const int r = idx / w, c = idx - r * w;
-            base[(long long)r * ldm + c] = Sb[c * R + pos2row[r]];
-        }
-        __syncthreads();
-        // This block's interchanges on the panel's other columns: at most 2w
-        // positions moved (pos2row[r] != r); their values are all read before
-        // any is written.
-        if (tid == 0) s_nmv = 0;
-        __syncthreads();
-        for (int r = tid; r < R; r += kPanelThreads)
-            if (pos2row[r] != r) mv[atomicAdd(&s_nmv, 1)] = (unsigned short)r;
-        __syncthreads();
-        {
-            const int nmv = s_nmv, nother = nb - w;
-            T val[kSwapPer];
-#pragma unroll
-            for (int u = 0; u < kSwapPer; ++u) {
-                const int idx = tid + u * kPanelThreads;
-                if (idx < nmv * nother) {
-                    const int q = idx / nother, oc = idx - q * nother;
-                    const int col = oc < jb ? oc : oc + w;
-                    val[u] = Mb[(long long)(k + jb + pos2row[mv[q]]) * ldm + k + col];
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < kSwapPer; ++u) {
-                const int idx = tid + u * kPanelThreads;
-                if (idx < nmv * nother) {
-                    const int q = idx / nother, oc = idx - q * nother;
-                    const int col = oc < jb ? oc : oc + w;
-                    Mb[(long long)(k + jb + mv[q]) * ldm + k + col] = val[u];
-                }
-            }
-        }
-        __syncthreads();
-        // Right-looking update of the panel columns [jb+w, nb): U12 rows by a
-        // forward substitution, then the trailing rows, each thread taking a
-        // 4 x 4 tile (per pivot column: 4 loads of L, one 4-wide load of U12,
-        // 16 multiply-adds); consecutive threads take consecutive column
-        // groups of the same rows, so the global accesses are contiguous.
-        const int ncr = nb - jb - w;
-        if (ncr > 0) {
-            T* rb = Mb + (long long)(k + jb) * ldm + (k + jb + w);
-            for (int col = tid; col < ncr; col += kPanelThreads) {
-                for (int c = 0; c < w; ++c) {
-                    T x = rb[(long long)c * ldm + col];
-                    const int pc = pos2row[c];
-                    for (int c2 = 0; c2 < c; ++c2) x -= Sb[c2 * R + pc] * Xs[c2 * kMaxNB + col];
-                    Xs[c * kMaxNB + col] = x;
-                    rb[(long long)c * ldm + col] = x;
-                }
-            }
-            __syncthreads();
-            const int rg = (R - w + 3) >> 2, cg = (ncr + 3) >> 2;
-            const bool vec = sizeof(T) == 4 && ((reinterpret_cast<uintptr_t>(rb) & 15) == 0) && (ldm & 3) == 0;
-            for (int item = tid; item < rg * cg; item += kPanelThreads) {
-                const int gi = item / cg, gc = item - gi * cg;
-                const int r0 = w + 4 * gi, c0 = 4 * gc;
-                int src[4];
-                T acc[4][4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int r = r0 + u;
-                    src[u] = pos2row[r < R ? r : w];
-                    T* rowp = rb + (long long)r * ldm + c0;
-                    if (r < R && vec && c0 + 3 < ncr) {
-                        const float4 v4 = *reinterpret_cast<const float4*>(rowp);
-                        acc[u][0] = T(v4.x); acc[u][1] = T(v4.y); acc[u][2] = T(v4.z); acc[u][3] = T(v4.w);
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) acc[u][v] = (r < R && c0 + v < ncr) ? rowp[v] : T(0);
-                    }
-                }
-                for (int c = 0; c < w; ++c) {
-                    T a[4], bv[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) a[u] = Sb[c * R + src[u]];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) bv[v] = Xs[c * kMaxNB + c0 + v];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) acc[u][v] -= a[u] * bv[v];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int r = r0 + u;
-                    if (r >= R) break;
-                    T* rowp = rb + (long long)r * ldm + c0;
-                    if (vec && c0 + 3 < ncr) {
-                        *reinterpret_cast<float4*>(rowp) =
-                            make_float4(float(acc[u][0]), float(acc[u][1]), float(acc[u][2]), float(acc[u][3]));
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < 4; ++v)
-                            if (c0 + v < ncr) rowp[v] = acc[u][v];
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-
-    // Row permutation of the step: position r holds the old row perm[r].
-    int* pb = perm + box * sP;
-    for (int r = tid; r < R0; r += kPanelThreads) pb[r] = r;
-    __syncthreads();
-    if (tid == 0)
-        for (int i = 0; i < nb; ++i) {
-            const int a = i, bb = swp[i];
-            if (a != bb) { const int t = pb[a]; pb[a] = pb[bb]; pb[bb] = t; }
-        }
-    if (tid == 0 && s_sing && status[box] == 0) status[box] = HPS_ESINGULAR;
-
-    // Inverses of the diagonal blocks, L11^{-1} and U11^{-1}, by blocks.
-    int Pd = 16;
-    while (Pd < nb) Pd *= 2;
-    T* Ap = Sb;                 // Pd x Pd, padded with the identity
-    T* X = Sb + Pd * Pd;        // the inverse
-    for (int idx = tid; idx < Pd * Pd; idx += kPanelThreads) {
-        const int r = idx / Pd, c = idx - r * Pd;
-        Ap[idx] = (r < nb && c < r) ? Mb[(long long)(k + r) * ldm + k + c] : T(0);
-        X[idx] = T(0);
-    }
-    __syncthreads();
-    tri_inverse<T>(Ap, X, Pd, true, tid);
-    T* Fb = Ftop + box * sF;
-    for (int idx = tid; idx < nb * nb; idx += kPanelThreads) {
-        const int r = idx / nb, c = idx - r * nb;
-        Fb[r * ldf + c] = -X[r * Pd + c];
-    }
-    __syncthreads();
-    for (int idx = tid; idx < Pd * Pd; idx += kPanelThreads) {
-        const int r = idx / Pd, c = idx - r * Pd;
-        Ap[idx] = (r < nb && c >= r && c < nb) ? Mb[(long long)(k + r) * ldm + k + c] : (r == c && r >= nb ? T(1) : T(0));
-        X[idx] = T(0);
-    }
-    __syncthreads();
-    tri_inverse<T>(Ap, X, Pd, false, tid);
-    T* Bb = Btop + box * sB;
-    for (int idx = tid; idx < nb * nb; idx += kPanelThreads) {
-        const int r = idx / nb, c = idx - r * nb;
-        Bb[r * ldb + c] = -X[r * Pd + c];
     }
 }
 
@@ -1622,37 +1286,6 @@ void launch_load_rhs(const Geometry& g, int nbox, int rhs_kind, int nrhs, const 
 }
 
 template <typename T>
-void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int ib,
-                  int* perm, long long sP, T* Ftop, long long ldf, long long sF,
-                  T* Btop, long long ldb, long long sB, int* status, const int* skip,
-                  int nbox, cudaStream_t st)
-{
-    static size_t dyn_max = 0;
-    if (!dyn_max) {
-        cudaFuncAttributes fa{};
-        cudaFuncGetAttributes(&fa, k_panel<T>);
-        dyn_max = 227 * 1024 - fa.sharedSizeBytes;
-        cudaFuncSetAttribute(k_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_max);
-    }
-    // Widest inner block (<= 32 columns, power of two) whose rows fit in what
-    // is left of shared memory; the panel shrinks as k grows, so later steps
-    // take wider blocks.  The plan's ib is the width of the first step.
-    const size_t R0 = (size_t)(n - k);
-    ib = 32;
-    while (ib > 1 && (size_t)ib * R0 * sizeof(T) + R0 * 5 > dyn_max) ib >>= 1;
-    if (ib > nb) ib = nb;
-    const size_t s1 = (size_t)ib * R0 * sizeof(T) + R0 * 5;
-    int Pd = 16;
-    while (Pd < nb) Pd *= 2;
-    const size_t s2 = (size_t)2 * Pd * Pd * sizeof(T);   // the padded triangle and its inverse
-    const size_t smem = s1 > s2 ? s1 : s2;
-    prof_begin(KC_PANEL, st);
-    k_panel<T><<<nbox, kPanelThreads, smem, st>>>(M, ldm, sM, n, k, nb, ib, perm, sP, Ftop, ldf, sF,
-                                                  Btop, ldb, sB, status, skip);
-    prof_end(KC_PANEL, st, (double)nbox * (n - k) * (double)nb * nb, (double)nbox * 2.0 * (n - k) * nb * sizeof(T));
-}
-
-template <typename T>
 void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c0, int ncols,
                    const int* perm, long long sP, T* W, T* G, long long ldg, long long sG,
                    const int* skip, int nbox, cudaStream_t st)
@@ -1982,12 +1615,6 @@ template void launch_load_rhs<float>(const Geometry&, int, int, int, const doubl
                                      long long, int*, cudaStream_t, const double*);
 template void launch_load_rhs<double>(const Geometry&, int, int, int, const double*, long long, double*, long long,
                                       long long, int*, cudaStream_t, const double*);
-template void launch_panel<float>(float*, long long, long long, int, int, int, int, int*, long long, float*,
-                                  long long, long long, float*, long long, long long, int*, const int*, int,
-                                  cudaStream_t);
-template void launch_panel<double>(double*, long long, long long, int, int, int, int, int*, long long, double*,
-                                   long long, long long, double*, long long, long long, int*, const int*, int,
-                                   cudaStream_t);
 template void launch_gather<float>(const float*, long long, long long, int, int, int, int, const int*, long long,
                                    float*, float*, long long, long long, const int*, int, cudaStream_t);
 template void launch_gather<double>(const double*, long long, long long, int, int, int, int, const int*,
