@@ -2,9 +2,9 @@
 // with partial pivoting) and the inverses of its diagonal blocks.
 //
 // A panel is the columns [k, k + nb) of rows [k, n) of one box.  A cluster of
-// C CTAs (256 threads each) takes one box; row r belongs for the whole panel
-// to thread r mod 256 of CTA (r / 256) mod C, and rows never move while the
-// panel is factored.  The panel goes left to right in blocks of IB columns
+// C CTAs (256 threads each) takes one box, groups of 32 rows dealt out to the
+// CTAs and then to their warps; a row belongs to one thread for the whole
+// panel, and rows never move while it is factored.  The panel goes left to right in blocks of IB columns
 // that a thread holds for its RPT rows in registers:
 //   1. load the block; for each earlier block: the rows that were its pivots
 //      hand their entries over, the block's unit triangle (its inverse, kept)
@@ -15,10 +15,11 @@
 //      CTAs' offers are exchanged through distributed shared memory and a
 //      cluster barrier), and every thread eliminates with the winning row
 //      from shared memory;
-//   3. multipliers of the rows still active go back to the matrix.
-// At the end the first CTA places the pivot rows on top, moves the rows they
-// displaced and writes the step's permutation (perm[r]: the old row at
-// position r, as a sequence of row swaps would give it).
+//   3. multipliers of the rows still active go to a scratch block by columns,
+//      where a warp reads and writes whole lines.
+// At the end every row goes to its place in the matrix: pivot rows on top, rows
+// they displaced where the row swaps would have taken them; perm[r] is the old
+// row at position r.
 //
 // What bounds it: with many boxes the multiply-adds of the elimination
 // (R nb^2 / 2 per box: the FP32 pipes at 128 a clock, the FP64 pipes at 2);
@@ -28,6 +29,7 @@
 // a panel in shared memory took two reads and a write per multiply-add.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "hps_internal.h"
 #include "hps_ptx.cuh"
@@ -73,6 +75,10 @@ __device__ __forceinline__ void remote_store(uint32_t a, unsigned long long v)
 {
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
+__device__ __forceinline__ void remote_store(uint32_t a, unsigned v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
 __device__ __forceinline__ void remote_store(uint32_t a, int v)
 {
     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
@@ -80,35 +86,83 @@ __device__ __forceinline__ void remote_store(uint32_t a, int v)
 
 // Pivot key of a value: larger for larger magnitudes, 1 for a NaN (taken only
 // when nothing else is left); 0 is kept for rows that are no candidates.
-__device__ __forceinline__ unsigned long long pivot_key(float x)
+template <typename T>
+using PivotKey = typename std::conditional<sizeof(T) == 4, unsigned, unsigned long long>::type;
+__device__ __forceinline__ unsigned pivot_key(float x)
 {
-    return x != x ? 1ull : (unsigned long long)(__float_as_uint(x) & 0x7FFFFFFFu) + 2ull;
+    return x != x ? 1u : (__float_as_uint(x) & 0x7FFFFFFFu) + 2u;
 }
 __device__ __forceinline__ unsigned long long pivot_key(double x)
 {
-    return x != x ? 1ull : ((unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull) + 2ull;
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+    return u > 0x7FF0000000000000ull ? 1ull : u + 2ull;
 }
 
 // Largest key over the lanes and, among its holders, the lowest row; true on
-// the lane that holds it.  FP32 keys fit 32 bits.
-template <typename T>
-__device__ __forceinline__ bool warp_argmax(unsigned long long& key, int& row)
+// the lane that holds it.
+__device__ __forceinline__ bool warp_argmax(unsigned& key, int& row)
 {
-    bool mine = key != 0;
-    if constexpr (sizeof(T) == 4) {
-        const unsigned k = (unsigned)key, m = __reduce_max_sync(0xffffffffu, k);
-        mine = mine && k == m;
-        key = m;
-    } else {
-        const unsigned h = (unsigned)(key >> 32), mh = __reduce_max_sync(0xffffffffu, h);
-        const unsigned l = h == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, l);
-        mine = mine && h == mh && l == ml;
-        key = ((unsigned long long)mh << 32) | ml;
-    }
+    const unsigned m = __reduce_max_sync(0xffffffffu, key);
+    bool mine = key != 0 && key == m;
+    key = m;
     const int r = __reduce_min_sync(0xffffffffu, mine ? row : INT_MAX);
     mine = mine && row == r;
     row = r;
     return mine;
+}
+__device__ __forceinline__ bool warp_argmax(unsigned long long& key, int& row)
+{
+    const unsigned h = (unsigned)(key >> 32), mh = __reduce_max_sync(0xffffffffu, h);
+    const unsigned l = h == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, l);
+    bool mine = key != 0 && h == mh && l == ml;
+    key = ((unsigned long long)mh << 32) | ml;
+    const int r = __reduce_min_sync(0xffffffffu, mine ? row : INT_MAX);
+    mine = mine && row == r;
+    row = r;
+    return mine;
+}
+
+// 1 / x.  FP64: on the integer pipe (a division is ten dependent operations of
+// 64 clocks a warp on the FP64 pipe): y, 1 / m to 22 bits from FP32, then
+// y (1 + e + e^2) with e = 1 - m y in fixed point, |e|^3 below 2^-66, rounded
+// once; below 0.51 units in the last place.
+__device__ __forceinline__ float reciprocal(float x) { return 1.0f / x; }
+__device__ __forceinline__ double reciprocal(double x)
+{
+    const uint64_t u = (uint64_t)__double_as_longlong(x);
+    const int ex = (int)(u >> 52) & 0x7ff;
+    if (ex - 1 > 2042) return 1.0 / x;   // subnormal results, infinities, NaN
+    if (ex == 0) return 1.0 / x;
+    const uint64_t M = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;             // m 2^52
+    const float mf = __uint_as_float(0x3F800000u | (uint32_t)((M >> 29) & 0x7FFFFFu));
+    const uint32_t yb = __float_as_uint(__frcp_rn(mf));
+    const uint32_t Y = yb >= 0x3F800000u ? 0x80000000u : ((yb & 0x7FFFFFu) | 0x800000u) << 7;   // y 2^31
+    const long long E = -(long long)(M * (uint64_t)Y);                               // e 2^83 (2^83 = 0 mod 2^64)
+    const long long t = __mul64hi(E, (long long)((uint64_t)Y << 12));                // y e 2^62
+    const long long R = (long long)((uint64_t)Y << 31) + t + (__mul64hi(t, E) >> 19);
+    const uint64_t mant = (uint64_t)(R + 256) >> 9;
+    return __longlong_as_double((long long)((u & 0x8000000000000000ull) | (((uint64_t)(2044 - ex) << 52) + mant)));
+}
+
+// a -= l u over a row; FP32 two entries an instruction (the same rounding).
+template <int N>
+__device__ __forceinline__ void sub_row(float (&a)[N], float l, const float (&u)[N])
+{
+    const float m = -l;
+#pragma unroll
+    for (int i = 0; i < N; i += 2)
+        asm("{\n\t.reg .b64 x, y, z;\n\t"
+            "mov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %2};\n\tmov.b64 z, {%3, %4};\n\t"
+            "fma.rn.f32x2 x, y, z, x;\n\t"
+            "mov.b64 {%0, %1}, x;\n\t}"
+            : "+f"(a[i]), "+f"(a[i + 1])
+            : "f"(m), "f"(u[i]), "f"(u[i + 1]));
+}
+template <int N>
+__device__ __forceinline__ void sub_row(double (&a)[N], double l, const double (&u)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] -= l * u[i];
 }
 
 template <typename T, int N>
@@ -139,11 +193,21 @@ __device__ __forceinline__ void store_row(T* s, const T (&d)[N])
     }
 }
 
+// 16-byte unit q of row r in a warp's tile of 32 rows of 64 bytes, swizzled so
+// that neither a lane per row nor four lanes per row meet in a bank.
+template <typename T>
+__device__ __forceinline__ float4* tile_unit(T* tile, int r, int q)
+{
+    return reinterpret_cast<float4*>(tile) + r * 4 + (q ^ ((r >> 1) & 3));
+}
+
 template <typename T>
 struct PanelArgs {
     T* M;
     long long ldm, sM;
     int n, k, nb;
+    T* Lt;           // scratch [nb][n - k] per box: the multipliers by columns while the panel is factored
+    long long sL;
     int* perm;
     long long sP;
     int* status;
@@ -153,16 +217,16 @@ struct PanelArgs {
 // Shared memory of a panel CTA.
 template <typename T, int IB>
 struct PanelSmem {
+    alignas(16) T tile[PW][32 * 64 / sizeof(T)];   // per warp: 32 rows of 64 bytes between row and column order
     alignas(16) T inv[kMaxNB / IB][IB][IB];        // inverses of the blocks' unit lower triangles
     alignas(16) T raw[2][IB][IB], u[IB][IB];       // a block's pivot rows before (alternating: a CTA may run one
                                                    // block ahead of its cluster) and after its triangle
     alignas(16) T cand[2][PW][IB];                 // the warps' offers
     alignas(16) T offer[2][kMaxCluster][IB];       // the CTAs' offers
-    unsigned long long ckey[2][PW], okey[2][kMaxCluster];
+    PivotKey<T> ckey[2][PW], okey[2][kMaxCluster];
     int crow[2][PW], orow[2][kMaxCluster];
     int prow[kMaxNB];                              // row chosen for each column
     int pp[kMaxNB];                                // position it had been swapped to
-    int moved_from[kMaxNB], moved_to[kMaxNB], nmoved;
     unsigned char is_pivot[kMaxNB];
     int sing;
 };
@@ -186,35 +250,73 @@ k_panel(const PanelArgs<T> a)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R0 = a.n - a.k;
     T* P = a.M + box * a.sM + (long long)a.k * a.ldm + a.k;   // the panel's corner
-    auto row_of = [&](int rr) { return (rr * C + rank) * PT + tid; };
+    auto row_of = [&](int rr) { return ((rr * PW + warp) * C + rank) * 32 + lane; };
+    // the warp's row groups that exist (all of a group's lanes may still be past the last row)
+    const int nrr = min(RPT, max(0, ((R0 + 31) / 32 - rank - warp * C + PW * C - 1) / (PW * C)));
 
     int pidx[RPT];   // column whose pivot the row became; -1 active, -2 no such row
 #pragma unroll
     for (int rr = 0; rr < RPT; ++rr) pidx[rr] = row_of(rr) < R0 ? -1 : -2;
     if (tid < kMaxNB) s.is_pivot[tid] = 0;
-    if (tid == 0) { s.sing = 0; s.nmoved = 0; }
+    if (tid == 0) s.sing = 0;
     if (C > 1) cluster_sync();   // every CTA of the cluster runs before its shared memory is written
 
+    constexpr int CU = 16 / sizeof(T), CW = 4 * CU;   // entries of a 16-byte unit and of a 64-byte row piece
+    T* tile = s.tile[warp];
+    T* Lt = a.Lt + box * a.sL;
     T x[RPT][IB];
     for (int b = 0; b < nblk; ++b) {
         const int jb = b * IB, w = min(IB, nb - jb);
-        // 1. the block's entries, brought up to date
+        // 1. the block's entries, brought up to date.  Rows are read 64 bytes at a
+        // time by four lanes each (a lane per row would touch 32 lines an
+        // instruction) and turned through the warp's tile.
 #pragma unroll
         for (int rr = 0; rr < RPT; ++rr) {
 #pragma unroll
             for (int c = 0; c < IB; ++c) x[rr][c] = T(0);
-            if (pidx[rr] != -2) {
-                const T* src = P + (long long)row_of(rr) * a.ldm + jb;
-                if (w == IB) load_row<T, IB>(x[rr], src);
-                else {
+            if (rr >= nrr) continue;
+            const int row0 = row_of(rr) - lane;
+            if (w == IB) {
 #pragma unroll
-                    for (int c = 0; c < IB; ++c)
-                        if (c < w) x[rr][c] = src[c];
+                for (int h = 0; h < IB / CW; ++h) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = 8 * i + (lane >> 2);
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (row0 + r < R0)
+                            v = *reinterpret_cast<const float4*>(P + (long long)(row0 + r) * a.ldm + jb + h * CW + (lane & 3) * CU);
+                        *tile_unit(tile, r, lane & 3) = v;
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 v = *tile_unit(tile, lane, q);
+                        const T* e = reinterpret_cast<const T*>(&v);
+#pragma unroll
+                        for (int t = 0; t < CU; ++t) x[rr][h * CW + q * CU + t] = e[t];
+                    }
+                    __syncwarp();
                 }
+            } else if (pidx[rr] != -2) {
+                const T* src = P + (long long)row_of(rr) * a.ldm + jb;
+#pragma unroll
+                for (int c = 0; c < IB; ++c)
+                    if (c < w) x[rr][c] = src[c];
             }
         }
         for (int e = 0; e < b; ++e) {
             const int je = e * IB;
+            constexpr int JC = RPT * (int)sizeof(T) >= 32 ? 2 : 4;   // multipliers read ahead per row
+            T l[RPT][JC];
+            auto load_l = [&](int j0) {
+#pragma unroll
+                for (int rr = 0; rr < RPT; ++rr) {
+                    const bool on = pidx[rr] == -1 || pidx[rr] >= je + IB;
+#pragma unroll
+                    for (int j = 0; j < JC; ++j) l[rr][j] = on ? Lt[(long long)(je + j0 + j) * R0 + row_of(rr)] : T(0);
+                }
+            };
+            load_l(0);
 #pragma unroll
             for (int rr = 0; rr < RPT; ++rr)
                 if (pidx[rr] >= je && pidx[rr] < je + IB) {
@@ -241,111 +343,126 @@ k_panel(const PanelArgs<T> a)
                 LU[(je + i) * ldl + jb + c] = v;
             }
             __syncthreads();
-            constexpr int JC = 16 / sizeof(T);   // multipliers read at a time (16 bytes)
 #pragma unroll 1
             for (int j0 = 0; j0 < IB; j0 += JC) {
-                T l[RPT][JC];
+                T lc[RPT][JC];
 #pragma unroll
-                for (int rr = 0; rr < RPT; ++rr) {
-                    const bool on = pidx[rr] == -1 || pidx[rr] >= je + IB;
+                for (int rr = 0; rr < RPT; ++rr)
 #pragma unroll
-                    for (int j = 0; j < JC; ++j) l[rr][j] = T(0);
-                    if (on) load_row<T, JC>(l[rr], P + (long long)row_of(rr) * a.ldm + je + j0);
-                }
+                    for (int j = 0; j < JC; ++j) lc[rr][j] = l[rr][j];
+                if (j0 + JC < IB) load_l(j0 + JC);
 #pragma unroll
                 for (int j = 0; j < JC; ++j) {
                     T uv[IB];
                     load_row<T, IB>(uv, s.u[j0 + j]);
 #pragma unroll
                     for (int rr = 0; rr < RPT; ++rr)
-#pragma unroll
-                        for (int c = 0; c < IB; ++c) x[rr][c] -= l[rr][j] * uv[c];
+                        if (rr < nrr) sub_row(x[rr], lc[rr][j], uv);
                 }
             }
         }
-        // 2. factor the block
+        // 2. factor the block.  A row's entries move one register down per
+        // column, so that the column at hand is always x[.][0] and the loop stays
+        // small (unrolled over the columns it outgrows the instruction cache);
+        // the multipliers fill the registers that come free at the end.
+#pragma unroll 1
+        for (int c = 0; c < w; ++c) {
+            const int cur = c & 1;
+            PivotKey<T> key = 0;
+            int row = INT_MAX, brr = 0;
 #pragma unroll
-        for (int c = 0; c < IB; ++c) {
-            if (c < w) {
-                const int cur = c & 1;
-                unsigned long long key = 0;
-                int row = INT_MAX, brr = 0;
+            for (int rr = 0; rr < RPT; ++rr) {
+                const PivotKey<T> kk = pidx[rr] == -1 ? pivot_key(x[rr][0]) : PivotKey<T>(0);
+                if (kk > key) { key = kk; row = row_of(rr); brr = rr; }
+            }
+            if (warp_argmax(key, row)) {
 #pragma unroll
-                for (int rr = 0; rr < RPT; ++rr) {
-                    const unsigned long long kk = pidx[rr] == -1 ? pivot_key(x[rr][c]) : 0ull;
-                    if (kk > key) { key = kk; row = row_of(rr); brr = rr; }
+                for (int rr = 0; rr < RPT; ++rr)
+                    if (rr == brr) store_row<T, IB>(s.cand[cur][warp], x[rr]);
+            }
+            if (lane == 0) { s.ckey[cur][warp] = key; s.crow[cur][warp] = row; }
+            __syncthreads();
+            // the CTA's best (every warp finds it for itself)
+            key = lane < PW ? s.ckey[cur][lane] : PivotKey<T>(0);
+            row = lane < PW ? s.crow[cur][lane] : INT_MAX;
+            unsigned who = __ballot_sync(0xffffffffu, warp_argmax(key, row));
+            const T* pv = s.cand[cur][who ? __ffs((int)who) - 1 : 0];
+            if (C > 1) {
+                if (warp == 0) {
+                    for (int e = lane; e < C * IB; e += 32) {
+                        const int d = e / IB, cc = e - d * IB;
+                        remote_store(remote_addr(&s.offer[cur][rank][cc], (unsigned)d), pv[cc]);
+                    }
+                    if (lane < C) {
+                        remote_store(remote_addr(&s.okey[cur][rank], (unsigned)lane), key);
+                        remote_store(remote_addr(&s.orow[cur][rank], (unsigned)lane), row);
+                    }
                 }
-                const bool mine = warp_argmax<T>(key, row);
-                if (mine) {
+                cluster_sync();
+                key = lane < C ? s.okey[cur][lane] : PivotKey<T>(0);
+                row = lane < C ? s.orow[cur][lane] : INT_MAX;
+                who = __ballot_sync(0xffffffffu, warp_argmax(key, row));
+                pv = s.offer[cur][who ? __ffs((int)who) - 1 : 0];
+            }
+            T piv = pv[0];
+            if (piv == T(0)) {   // exactly singular: record it and keep the arithmetic finite
+                if (tid == 0) s.sing = 1;
+                piv = T(1);
+            }
+            const T rinv = reciprocal(piv);
+            if (tid < IB) LU[(jb + c) * ldl + jb + ((tid + c) & (IB - 1))] = pv[tid];
+            if (tid == 32) {
+                s.prow[jb + c] = row;
+                if (row < nb) s.is_pivot[row] = 1;
+                int pos = row;   // follow the swaps that moved the row before
+                while (pos < jb + c) pos = s.pp[pos];
+                s.pp[jb + c] = pos;
+            }
+            T l[RPT];
+#pragma unroll
+            for (int rr = 0; rr < RPT; ++rr) {
+                if (row_of(rr) == row) pidx[rr] = jb + c;
+                l[rr] = x[rr][0] * rinv;
+            }
+            constexpr int PC = 16 / sizeof(T);   // pivot-row entries read at a time (16 bytes)
+#pragma unroll
+            for (int i0 = 0; i0 < IB; i0 += PC) {
+                T p[PC];
+                load_row<T, PC>(p, pv + i0);
+#pragma unroll
+                for (int u = 0; u < PC; ++u) {
+                    const int i = i0 + u;
+                    if (i == 0) continue;
+                    // entries past the block's columns are multipliers: left as they are
+                    const bool col = i < IB - c;
+                    const T pu = col ? p[u] : T(0);
 #pragma unroll
                     for (int rr = 0; rr < RPT; ++rr)
-                        if (rr == brr) store_row<T, IB>(s.cand[cur][warp], x[rr]);
-                }
-                if (lane == 0) { s.ckey[cur][warp] = key; s.crow[cur][warp] = row; }
-                __syncthreads();
-                // the CTA's best (every warp finds it for itself)
-                key = lane < PW ? s.ckey[cur][lane] : 0ull;
-                row = lane < PW ? s.crow[cur][lane] : INT_MAX;
-                const unsigned who = __ballot_sync(0xffffffffu, warp_argmax<T>(key, row));
-                int best = who ? __ffs((int)who) - 1 : 0;
-                const T* pv = s.cand[cur][best];
-                if (C > 1) {
-                    if (warp == 0) {
-                        for (int e = lane; e < C * IB; e += 32) {
-                            const int d = e / IB, cc = e - d * IB;
-                            remote_store(remote_addr(&s.offer[cur][rank][cc], (unsigned)d), pv[cc]);
+                        if (rr < nrr) {
+                            if constexpr (sizeof(T) == 4) x[rr][i - 1] = x[rr][i] - l[rr] * pu;
+                            else x[rr][i - 1] = col ? x[rr][i] - l[rr] * pu : x[rr][i];
                         }
-                        if (lane < C) {
-                            remote_store(remote_addr(&s.okey[cur][rank], (unsigned)lane), key);
-                            remote_store(remote_addr(&s.orow[cur][rank], (unsigned)lane), row);
-                        }
-                    }
-                    cluster_sync();
-                    key = lane < C ? s.okey[cur][lane] : 0ull;
-                    row = lane < C ? s.orow[cur][lane] : INT_MAX;
-                    const unsigned whoc = __ballot_sync(0xffffffffu, warp_argmax<T>(key, row));
-                    best = whoc ? __ffs((int)whoc) - 1 : 0;
-                    pv = s.offer[cur][best];
-                }
-                T p[IB];
-                load_row<T, IB>(p, pv);
-                T piv = p[c];
-                if (piv == T(0)) {   // exactly singular: record it and keep the arithmetic finite
-                    if (tid == 0) s.sing = 1;
-                    piv = T(1);
-                }
-                const T rinv = T(1) / piv;
-                if (tid < IB) LU[(jb + c) * ldl + jb + tid] = pv[tid];
-                if (tid == 32) {
-                    s.prow[jb + c] = row;
-                    if (row < nb) s.is_pivot[row] = 1;
-                    int pos = row;   // follow the swaps that moved the row before
-                    while (pos < jb + c) pos = s.pp[pos];
-                    s.pp[jb + c] = pos;
-                }
-#pragma unroll
-                for (int rr = 0; rr < RPT; ++rr) {
-                    if (row_of(rr) == row) pidx[rr] = jb + c;
-                    if (pidx[rr] == -1) {
-                        const T l = x[rr][c] * rinv;
-                        x[rr][c] = l;
-#pragma unroll
-                        for (int cc = c + 1; cc < IB; ++cc) x[rr][cc] -= l * p[cc];
-                    }
                 }
             }
+#pragma unroll
+            for (int rr = 0; rr < RPT; ++rr) x[rr][IB - 1] = l[rr];
         }
-        // 3. multipliers of the active rows
+        for (int c = w; c < IB; ++c) {   // a ragged block: turn the multipliers to the front
+#pragma unroll
+            for (int rr = 0; rr < RPT; ++rr) {
+                const T l = x[rr][0];
+#pragma unroll
+                for (int i = 1; i < IB; ++i) x[rr][i - 1] = x[rr][i];
+                x[rr][IB - 1] = l;
+            }
+        }
+        // 3. multipliers of the active rows, by columns
 #pragma unroll
         for (int rr = 0; rr < RPT; ++rr)
             if (pidx[rr] == -1) {
-                T* dst = P + (long long)row_of(rr) * a.ldm + jb;
-                if (w == IB) store_row<T, IB>(dst, x[rr]);
-                else {
 #pragma unroll
-                    for (int c = 0; c < IB; ++c)
-                        if (c < w) dst[c] = x[rr][c];
-                }
+                for (int c = 0; c < IB; ++c)
+                    if (c < w) Lt[(long long)(jb + c) * R0 + row_of(rr)] = x[rr][c];
             }
         __syncthreads();
         // the block's unit triangle inverted: a column per lane, each entry
@@ -363,33 +480,61 @@ k_panel(const PanelArgs<T> a)
         }
         __syncthreads();
     }
-    __threadfence();
     if (C > 1) cluster_sync();   // every row's multipliers are in memory; no distributed access follows
     else __syncthreads();
+
+    // Every row that became no pivot goes to its place: below the panel's top
+    // it stays, and one that a pivot displaced from the top moved to where that
+    // pivot had been, on from there if a later column took that place too.
+    int* pb = a.perm + box * a.sP;
+    for (int rr = 0; rr < nrr; ++rr) {
+        const int row = row_of(rr);
+        int pos = -1;
+        if (row < R0 && (row >= nb || !s.is_pivot[row])) {
+            bool pivot = false;
+            if (row >= nb) {
+#pragma unroll
+                for (int q = 0; q < RPT; ++q)
+                    if (q == rr) pivot = pidx[q] >= 0;
+            }
+            if (!pivot) {
+                pos = row;
+                while (pos < nb) pos = s.pp[pos];
+                pb[pos] = row;
+            }
+        }
+        for (int c0 = 0; c0 < nb; c0 += CW) {
+            if (c0 + CW <= nb) {
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float4 v;
+                    T* e = reinterpret_cast<T*>(&v);
+#pragma unroll
+                    for (int t = 0; t < CU; ++t) e[t] = pos >= 0 ? Lt[(long long)(c0 + q * CU + t) * R0 + row] : T(0);
+                    *tile_unit(tile, lane, q) = v;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = 8 * i + (lane >> 2), to = __shfl_sync(0xffffffffu, pos, r);
+                    if (to >= 0)
+                        *reinterpret_cast<float4*>(P + (long long)to * a.ldm + c0 + (lane & 3) * CU) =
+                            *tile_unit(tile, r, lane & 3);
+                }
+            } else if (pos >= 0) {
+                for (int c = c0; c < nb; ++c) P[(long long)pos * a.ldm + c] = Lt[(long long)c * R0 + row];
+            }
+        }
+    }
     if (rank != 0) return;
 
-    // Pivot rows' multipliers of earlier blocks into LU, and where the rows
-    // that they displaced from the top go: a row swapped to a position that a
-    // later column takes moves on with it.
+    // The pivot rows on top: their multipliers of earlier blocks join what LU holds.
     for (int idx = tid; idx < nb * ldl; idx += PT) {
-        const int j = idx / ldl, c = idx - j * ldl;
-        if (c < j / IB * IB) LU[idx] = __ldcg(P + (long long)s.prow[j] * a.ldm + c);
+        const int j = idx % nb, c = idx / nb;
+        if (c < j / IB * IB) LU[j * ldl + c] = __ldcg(Lt + (long long)c * R0 + s.prow[j]);
     }
-    if (tid < nb && !s.is_pivot[tid]) {
-        int pos = tid;
-        while (pos < nb) pos = s.pp[pos];
-        const int q = atomicAdd(&s.nmoved, 1);
-        s.moved_from[q] = tid;
-        s.moved_to[q] = pos;
-    }
-    int* pb = a.perm + box * a.sP;
-    for (int r = tid; r < R0; r += PT) pb[r] = r < nb ? s.prow[r] : r;
-    __syncthreads();
-    for (int idx = tid; idx < s.nmoved * nb; idx += PT) {
-        const int q = idx / nb, c = idx - q * nb;
-        P[(long long)s.moved_to[q] * a.ldm + c] = __ldcg(P + (long long)s.moved_from[q] * a.ldm + c);
-    }
-    if (tid < s.nmoved) pb[s.moved_to[tid]] = s.moved_from[tid];
+    if (tid < nb) pb[tid] = s.prow[tid];
     __syncthreads();
     for (int idx = tid; idx < nb * nb; idx += PT) {
         const int j = idx / nb, c = idx - j * nb;
@@ -563,9 +708,9 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
     }();
     (void)once;
     // Rows per thread and cluster size: the fewest waves of (chain of nb pivots
-    // + the elimination's issue), with the measured clocks of one pivot: about
-    // 500 alone, 1100 in a cluster, and per row of a thread 160 (FP32) or 5200
-    // (FP64) shared by the CTAs of an SM.
+    // + the elimination's issue).  Clocks of one pivot: about 500 alone and 1100
+    // in a cluster, and per group of 32 rows 25 (FP32) or 640 (FP64: 40
+    // multiply-adds of 64 clocks over four schedulers), shared by an SM's CTAs.
     const int R0 = n - k;
     int bi = 3, bc = kMaxCluster;
     double best = -1.0;
@@ -579,12 +724,14 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
             const long long ctas = (long long)nbox * c, slots = 152LL * sh.occ;
             const double waves = (double)((ctas + slots - 1) / slots);
             const double share = (double)std::min<long long>(sh.occ, (ctas + 151) / 152);
-            const double rows = (double)std::min((long long)sh.rpt, ((long long)R0 + PT * c - 1) / (PT * c));
-            const double cost = waves * ((c == 1 ? 500.0 : 1100.0) + share * rows * (sizeof(T) == 4 ? 160.0 : 5200.0));
+            const double groups = (double)((R0 + 32 * c - 1) / (32 * c));
+            const double cost = waves * ((c == 1 ? 500.0 : 1100.0) + share * groups * (sizeof(T) == 4 ? 25.0 : 640.0));
             if (best < 0 || cost < best) { best = cost; bi = i; bc = c; }
         }
     }
-    PanelArgs<T> a{M, ldm, sM, n, k, nb, perm, sP, status, skip};
+    // the multipliers' scratch is the step's F block, which the inverse and the
+    // product after this overwrite
+    PanelArgs<T> a{M, ldm, sM, n, k, nb, Ftop, sF, perm, sP, status, skip};
     prof_begin(KC_PANEL, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nbox * bc));
