@@ -31,7 +31,7 @@
 // 0..7-i of B, N = 32 (8 - i): the diagonals t land in consecutive TMEM
 // columns), and while they run every warp joins 32 x 8 outputs of the tile
 // before (TMEM holds two tiles of 8 x 32 columns, all 512).  A tile's 4096
-// outputs need 2176 tensor-core clocks, about 2000 clocks of integer issue and
+// outputs need 2176 tensor-core clocks, about 2500 clocks of issue and
 // 2048 clocks of FP64 adds, and move 64 KB of O: the three are balanced, with
 // HBM close behind at K = 64.  Measured against the CUDA-core FP64 product:
 // 512 boxes at p = 12 (DtN, particular and reconstruction) 1001 -> 147 ms for
@@ -58,7 +58,8 @@ constexpr uint32_t OFF_B = DG_S * A_PLANE, OFF_ST = OFF_B + 2 * B_BUF;
 constexpr size_t DG_SMEM = OFF_ST + DG_WARPS * STAGE + 1024;
 constexpr uint64_t DG_WAIT_NS = 2000000000ull;
 constexpr int E_MIN = 1;     // scale exponent of a row or column of zeros (subnormal entries count as zero)
-constexpr int E_BAD = 2047;  // an infinity or NaN in the row or column
+constexpr int E_BAD = 2047;  // an infinity or NaN in the row or column: its scale is then kept as E_NAN
+constexpr int E_NAN = 1 << 20;
 
 struct DgArgs {
     GemmArgs<double> g;
@@ -110,21 +111,51 @@ __device__ __forceinline__ void split4(const double (&x)[4], int E, unsigned cha
     }
 }
 
-// Sum of acc_t 2^(45 - 8 t) (unit 2^-57 of 2^(Ea + Eb)) rounded once to FP64 with its scale.
-__device__ __forceinline__ double join(const int (&a)[DG_S], int Ea, int Eb)
+// Sum of acc_t 2^(45 - 8 t) (unit 2^-57 of the scales' product 2^(E - 1016 ..))
+// rounded once to FP64.  The accumulators are turned to integers by adding
+// 1.5 2^23 (the conversion instruction runs at 16 lanes a clock and took 93 %
+// of the kernel's time): exact below 2^22, which holds for t <= 4 (the leading
+// digits are at most 64).  t = 5 is first cut to a multiple of 4, whose rest
+// joins t = 6, 7; those only need to be right to a fraction of the unit, so
+// their sum is taken in FP32 (an error below 2^-4 units).
+// E: biased exponents of the two scales, less 1016.  A result outside the
+// normal range (or of a row or column with an infinity or NaN) sets `odd`, and
+// finish_odd gives it; the common path has no branch, so that the eight joins
+// of a thread overlap.
+__device__ __forceinline__ double join(const float (&a)[DG_S], int E, int& eb_out)
 {
-    const int a01 = a[0] * 256 + a[1], a23 = a[2] * 256 + a[3], a45 = a[4] * 256 + a[5], a67 = a[6] * 256 + a[7];
-    long long V = (long long)a23 * (1 << 21) + ((long long)a45 * 32 + ((a67 + 1024) >> 11));
-    V += (long long)((unsigned long long)(long long)a01 << 37);
-    const uint64_t sgn = (uint64_t)V & 0x8000000000000000ull;
-    uint64_t u = sgn ? 0ull - (uint64_t)V : (uint64_t)V;
-    if (u == 0) return 0.0;
-    const int lz = __clzll((long long)u);
-    u <<= lz;
-    const uint64_t mant = (u >> 11) + ((u >> 10) & 1ull);
-    const int eb = Ea + Eb - lz - 1016;   // biased exponent - 1 (the leading bit of mant adds it)
-    if ((unsigned)eb > 2045u) return __longlong_as_double((long long)(sgn | (eb < 0 ? 0ull : 0x7FF0000000000000ull)));
-    return __longlong_as_double((long long)(sgn | (mant + ((uint64_t)eb << 52))));
+    constexpr float MG = 12582912.0f;   // 1.5 2^23, bits 0x4B400000
+    constexpr uint32_t MB = 0x4B400000u;
+    auto bits = [](float x) { return __float_as_uint(x); };
+    const float h = __fmaf_rn(a[5], 0.25f, MG);
+    const float r5 = __fmaf_rn(-4.0f, __fsub_rn(h, MG), a[5]);                        // -2 .. 2
+    const float lo = __fmaf_rn(r5, 256.0f, __fmaf_rn(a[7], 0.00390625f, a[6]));       // unit 2^-3
+    const int low = (int)(bits(__fmaf_rn(lo, 0.125f, MG)) - MB);
+    const uint32_t a01 = bits(__fadd_rn(a[0], MG)) * 256u + (bits(__fadd_rn(a[1], MG)) - MB * 257u);
+    const int a23 = (int)(bits(__fadd_rn(a[2], MG)) * 256u + (bits(__fadd_rn(a[3], MG)) - MB * 257u));
+    const int a45 = (int)(bits(__fadd_rn(a[4], MG)) * 64u + (bits(h) - MB * 65u));    // unit 2^7
+    long long V = (long long)a23 * (1 << 21) + ((long long)a45 * 128 + low);
+    V += (long long)((uint64_t)(a01 << 5) << 32);
+    const int sm = (int)(V >> 63);
+    uint64_t u = (uint64_t)((V ^ (long long)sm) - (long long)sm);
+    const int lz = __clzll((long long)u);              // 1 .. 63, 64 for zero
+    u <<= (lz - 1) & 63;
+    u += 512;                                          // the leading bit is bit 62: 53 bits stay
+    int eb = E - lz;
+    uint64_t r = (u >> 10) + ((uint64_t)(uint32_t)eb << 52);
+    r |= (uint64_t)((uint32_t)sm & 0x80000000u) << 32;
+    const bool zero = lz == 64 && E < (1 << 19);
+    eb_out = zero ? 0 : lz == 64 ? 4096 : eb;
+    return __longlong_as_double(zero ? 0ll : (long long)r);
+}
+
+// The rare results: `r` has the sign, E and eb are those of its join.
+__device__ __noinline__ double finish_odd(double r, int E, int eb)
+{
+    if ((unsigned)eb <= 2045u) return r;
+    if (E >= (1 << 19)) return __longlong_as_double(0x7FF8000000000000ll);   // an infinity or NaN went in
+    const long long sg = __double_as_longlong(r) & (long long)0x8000000000000000ull;
+    return __longlong_as_double(sg | (eb < 0 ? 0ll : 0x7FF0000000000000ll));
 }
 
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr)
@@ -151,7 +182,8 @@ k_digit_gemm(const DgArgs a)
     __shared__ uint32_t tmem_sh;
     __shared__ int rowE[DG_BM];
     __shared__ int rowsrc[DG_BM];   // source of the row: -1 zero, -2 no such row, -3 the row itself, else a row of W
-    __shared__ int colE[4][DG_BN];
+    __shared__ int colE[4][DG_BN];  // largest exponents of a tile's columns
+    __shared__ int colX[2][DG_BN];  // the same, less 1016, for the join
     const GemmArgs<double>& g = a.g;
     const int box = blockIdx.z;
     if (g.skip && g.skip[box]) return;
@@ -172,7 +204,7 @@ k_digit_gemm(const DgArgs a)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), 512);
-    if (tid < 4 * DG_BN) (&colE[0][0])[tid] = 0;
+    if (tid < 4 * DG_BN) (&colE[0][0])[tid] = E_MIN;
     if (tid < DG_BM) {
         const int r = m0 + tid;
         int s = -2;
@@ -219,12 +251,21 @@ k_digit_gemm(const DgArgs a)
             for (int u = 0; u < 4; ++u) e = max(e, exp_of(x[ps][u]));
 #pragma unroll
             for (int off = 8; off > 0; off >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
-            if (kg == 0) rowE[rl] = e;
+            if (kg == 0) rowE[rl] = e == E_BAD ? E_NAN : e;
             split4(x[ps], e, sp + rl * 128 + (((kg >> 1) ^ (rl & 7)) << 4) + ((kg & 1) << 3), A_PLANE);
         }
     }
     __syncthreads();
     const uint32_t tmem = tmem_sh;
+    // where this lane's eight rows of a joined block take their source: the row itself, a row of W, or nothing
+    uint32_t own = 0, other = 0, valid = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int s = rowsrc[(warp & 3) * 32 + 4 * u + (lane >> 3)];
+        own |= (uint32_t)(s == -3) << u;
+        other |= (uint32_t)(s >= 0) << u;
+        valid |= (uint32_t)(s != -2) << u;
+    }
     const int kch = max(1, (min(g.K, DG_K) + 15) / 16);
     bool ok = true;
 
@@ -233,10 +274,13 @@ k_digit_gemm(const DgArgs a)
             int e = max(max(exp_of(bx[0]), exp_of(bx[1])), max(exp_of(bx[2]), exp_of(bx[3])));
             atomicMax(&colE[i & 3][lane], e);
             __syncthreads();
-            e = max(colE[i & 3][lane], E_MIN);
+            e = colE[i & 3][lane];
             split4(bx, e, sp + OFF_B + (i & 1) * B_BUF + lane * 128 + (((warp >> 1) ^ (lane & 7)) << 4) + ((warp & 1) << 3),
                    B_PLANE);
-            if (warp == 0) colE[(i + 2) & 3][lane] = 0;
+            if (warp == 0) {
+                colE[(i + 2) & 3][lane] = E_MIN;
+                colX[i & 1][lane] = e == E_BAD ? E_NAN : e - 1016;
+            }
             if (i + 1 < cnt) load_b(t0 + i + 1);
             fence_proxy_async_smem();
             tc_fence_before();
@@ -261,14 +305,18 @@ k_digit_gemm(const DgArgs a)
         const int n0 = (t0 + j) * DG_BN + cg;
         const int col = n0 + (lane & 7);
         double src[8];
-        int rs[8];
+        const bool in = col < g.N;
+        double* Oc = O + (long long)(m0 + rq + (lane >> 3)) * g.ldo + col;
+        const long long ostep = 4 * g.ldo;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int rl = rq + 4 * u + (lane >> 3);
-            rs[u] = col < g.N ? rowsrc[rl] : -2;
             src[u] = 0.0;
-            if (rs[u] == -3) src[u] = O[(long long)(m0 + rl) * g.ldo + col];
-            else if (rs[u] >= 0) src[u] = W[(long long)rs[u] * g.ldw + col];
+            if (in && (own >> u & 1)) src[u] = Oc[u * ostep];
+        }
+        if (other && in) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (other >> u & 1) src[u] = W[(long long)rowsrc[rq + 4 * u + (lane >> 3)] * g.ldw + col];
         }
         if (ok && !mbar_try_wait(smem_u32(&tfull[buf]), (j >> 1) & 1)) {
             const uint64_t w0 = global_ns();
@@ -281,25 +329,31 @@ k_digit_gemm(const DgArgs a)
         for (int t = 0; t < DG_S; ++t)
             tmem_ld8(tmem + ((uint32_t)rq << 16) + (uint32_t)(buf * 256 + t * DG_BN + cg), v[t]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int Ea = rowE[rq + lane];
+        const int Ea = ok ? rowE[rq + lane] : E_NAN;
         double* st = reinterpret_cast<double*>(sp + OFF_ST + warp * STAGE);
+        int eb[8];
+        bool odd = false;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const int Eb = max(colE[j & 3][cg + c], E_MIN);
-            int q[DG_S];
+            float q[DG_S];
 #pragma unroll
-            for (int t = 0; t < DG_S; ++t) q[t] = __float2int_rn(__uint_as_float(v[t][c]));
-            double r = join(q, Ea, Eb);
-            if (Ea == E_BAD || Eb == E_BAD || !ok) r = __longlong_as_double(0x7FF8000000000000ll);
-            st[lane * 8 + (c ^ ((lane >> 1) & 7))] = r;
+            for (int t = 0; t < DG_S; ++t) q[t] = __uint_as_float(v[t][c]);
+            st[lane * 8 + (c ^ ((lane >> 1) & 7))] = join(q, Ea + colX[buf][cg + c], eb[c]);
+            odd |= (unsigned)eb[c] > 2045u;
+        }
+        if (odd) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                double& r = st[lane * 8 + (c ^ ((lane >> 1) & 7))];
+                r = finish_odd(r, Ea + colX[buf][cg + c], eb[c]);
+            }
         }
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int rl = 4 * u + (lane >> 3);
-            if (rs[u] != -2)
-                O[(long long)(m0 + rq + rl) * g.ldo + col] =
-                    fma(g.alpha, st[rl * 8 + ((lane & 7) ^ ((rl >> 1) & 7))], src[u]);
+            const double r = fma(g.alpha, st[rl * 8 + ((lane & 7) ^ ((rl >> 1) & 7))], src[u]);
+            if (in && (valid >> u & 1)) Oc[u * ostep] = r;
         }
         tc_fence_before();
     }
