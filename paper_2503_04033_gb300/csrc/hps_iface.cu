@@ -35,6 +35,7 @@
 #include <new>
 #include <vector>
 
+#include "hps_conv.cuh"
 #include "hps_iface.h"
 #include "hps_internal.h"
 
@@ -327,72 +328,95 @@ __global__ void k_if_down(const IfDesc* __restrict__ desc, const int* __restrict
 
 // O = [acc] O + alpha A B for a batch of small-N products (N = nrhs <= 16,
 // NC columns per pass), A in the storage type MT, B and O in FP64, sums in
-// FP64.  TPR threads share one output row (32 .. 256, sized to K so that each
-// thread reads a few elements of it) and a CTA of 256 threads takes 256 / TPR
-// rows: rows of A are read once, coalesced, with enough loads in flight per
-// SM whether a level has one merge or hundreds.  Partial sums are joined by
-// warp shuffles, across warps through shared memory.  A [M][K] (pitch lda);
-// B element (k, c) at k bk + c bc; O element (r, c) at r ok + c oc.
-template <int NC, int TPR, typename MT>
-__global__ void __launch_bounds__(256) k_if_mv(int Mr, int K, int N, const MT* __restrict__ A, long long lda,
+// FP64.  A warp takes four rows of A and reads 16 bytes of each per lane and
+// step, so that one read of B serves four rows and 16 loads are in flight; KS
+// warps of a CTA share the rows along K where a level has few of them, and
+// join their sums through shared memory.  FP32 entries are widened on the
+// integer pipe: the FP64 pipe, two multiply-adds per clock and SM, then has
+// one per entry and load, which bounds FP32 matrices at 2.5 TB/s (FP64 ones at
+// HBM).  A refined solve of 8 x 8 x 8 boxes at p = 12 (six sweeps): 56 -> 20 ms
+// against a thread group per row with the entries converted on the FP64 pipe.  A [M][K] (pitch lda); B element (k, c) at k bk + c bc; O element
+// (r, c) at r ok + c oc.  VEC: the rows of A start on 16 bytes.
+template <int NC, typename MT, bool VEC>
+__global__ void __launch_bounds__(256) k_if_mv(int Mr, int K, int N, int KS, const MT* __restrict__ A, long long lda,
                                                long long sA, const double* __restrict__ B, long long sB,
                                                long long bk, long long bc, double* __restrict__ O, long long sO,
                                                long long ok, long long oc, double alpha, int acc,
                                                const int* __restrict__ skip)
 {
-    constexpr int RPC = 256 / TPR, WPR = TPR / 32;
+    constexpr int RW = 4, U = 16 / sizeof(MT);   // rows of a warp, entries of a 16-byte load
     if (skip && *skip) return;
-    __shared__ double red[8][NC];
+    __shared__ double red[8][RW][NC];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t = threadIdx.x % TPR, rloc = threadIdx.x / TPR;
-    const int row = blockIdx.x * RPC + rloc;
-    const bool live = row < Mr;
-    const MT* Ar = A + (long long)blockIdx.y * sA + (long long)(live ? row : 0) * lda;
+    const int grp = warp / KS, part = warp - grp * KS;
+    const int row0 = (blockIdx.x * (8 / KS) + grp) * RW;
+    const MT* Ab = A + (long long)blockIdx.y * sA;
     const double* Bb = B + (long long)blockIdx.y * sB;
-    double* Or = O + (long long)blockIdx.y * sO + (long long)row * ok;
+    double* Ob = O + (long long)blockIdx.y * sO;
+    const MT* Ar[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) Ar[r] = Ab + (long long)min(row0 + r, Mr - 1) * lda;
     for (int c0 = 0; c0 < N; c0 += NC) {
-        double s[NC];
+        double s[RW][NC];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] = 0.0;
-        if (live) {
-#pragma unroll 4
-            for (int k = t; k < K; k += TPR) {
-                const double a = (double)Ar[k];
-                const double* Bk = Bb + (long long)k * bk + (long long)c0 * bc;
+        for (int r = 0; r < RW; ++r)
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (c0 + c < N) s[c] += a * Bk[c * bc];
-            }
-        }
+            for (int c = 0; c < NC; ++c) s[r][c] = 0.0;
+        if (row0 < Mr) {
+#pragma unroll 2
+            for (int k = (part * 32 + lane) * U; k < K; k += KS * 32 * U) {
+                MT av[RW][U];
+                double bv[U][NC];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
+                for (int r = 0; r < RW; ++r) {
+                    if (VEC && k + U <= K) {
+                        const float4 t = __ldg(reinterpret_cast<const float4*>(Ar[r] + k));
+                        const MT* e = reinterpret_cast<const MT*>(&t);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
-        }
-        if (WPR == 1) {
-            if (live) {
+                        for (int u = 0; u < U; ++u) av[r][u] = e[u];
+                    } else {
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (lane == c && c0 + c < N) {
-                        double* o = Or + (long long)(c0 + c) * oc;
-                        *o = (acc ? *o : 0.0) + alpha * s[c];
+                        for (int u = 0; u < U; ++u) av[r][u] = k + u < K ? Ar[r][k + u] : MT(0);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c)
+                        bv[u][c] = (k + u < K && c0 + c < N) ? Bb[(long long)(k + u) * bk + (long long)(c0 + c) * bc] : 0.0;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int r = 0; r < RW; ++r) {
+                        double a;
+                        if constexpr (sizeof(MT) == 4) a = hps::f2d(av[r][u]);
+                        else a = av[r][u];
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) s[r][c] += a * bv[u][c];
                     }
             }
-        } else {
-            if (lane == 0) {
+        }
 #pragma unroll
-                for (int c = 0; c < NC; ++c) red[warp][c] = s[c];
+        for (int r = 0; r < RW; ++r)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s[r][c] += __shfl_xor_sync(0xffffffffu, s[r][c], o);
+                if (lane == 0) red[warp][r][c] = s[r][c];
             }
-            __syncthreads();
-            if (live && t < NC && c0 + t < N) {
+        if (KS > 1) __syncthreads();
+        else __syncwarp();
+        if (part == 0 && lane < RW * NC) {
+            const int r = lane / NC, c = lane - r * NC;
+            if (row0 + r < Mr && c0 + c < N) {
                 double v = 0.0;
-#pragma unroll
-                for (int w = 0; w < WPR; ++w) v += red[rloc * WPR + w][t];
-                double* o = Or + (long long)(c0 + t) * oc;
+                for (int w = 0; w < KS; ++w) v += red[warp + w][r][c];
+                double* o = Ob + (long long)(row0 + r) * ok + (long long)(c0 + c) * oc;
                 *o = (acc ? *o : 0.0) + alpha * v;
             }
-            __syncthreads();
         }
+        if (KS > 1) __syncthreads();
+        else __syncwarp();
     }
 }
 
@@ -401,18 +425,29 @@ void launch_mv(int nn, int Mr, int N, int K, const MT* A, long long lda, long lo
                long long bk, long long bc, double* O, long long sO, long long ok, long long oc, double alpha, int acc,
                const int* skip, cudaStream_t st)
 {
-    // threads per row: about K / 8 elements each, 32 .. 256
-    int tpr = 32;
-    while (tpr < 256 && tpr * 8 < K) tpr *= 2;
-    const unsigned rows_per_cta = 256 / tpr;
-    dim3 grd((unsigned)((Mr + rows_per_cta - 1) / rows_per_cta), (unsigned)nn);
-#define IF_MV(TP) \
-    k_if_mv<NC, TP, MT><<<grd, 256, 0, st>>>(Mr, K, N, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip)
-    if (tpr == 32) IF_MV(32);
-    else if (tpr == 64) IF_MV(64);
-    else if (tpr == 128) IF_MV(128);
-    else IF_MV(256);
-#undef IF_MV
+    // Warps per row group: more while the level's rows leave SMs without eight
+    // CTAs' worth of warps and every warp still has a step of K.
+    int ks = 1;
+    while (ks < 8 && (long long)nn * Mr * ks < 152LL * 8 * 32 && K > ks * 32 * (int)(16 / sizeof(MT))) ks *= 2;
+    const int rows_per_cta = 32 / ks;
+    const bool vec = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && lda * sizeof(MT) % 16 == 0 && sA * sizeof(MT) % 16 == 0;
+    const dim3 grd((unsigned)((Mr + rows_per_cta - 1) / rows_per_cta), (unsigned)nn);
+    if (vec)
+        k_if_mv<NC, MT, true><<<grd, 256, 0, st>>>(Mr, K, N, ks, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip);
+    else
+        k_if_mv<NC, MT, false><<<grd, 256, 0, st>>>(Mr, K, N, ks, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip);
+}
+
+template <typename MT>
+void launch_mv_n(int nn, int Mr, int N, int K, const MT* A, long long lda, long long sA, const double* B, long long sB,
+                 long long bk, long long bc, double* O, long long sO, long long ok, long long oc, double alpha, int acc,
+                 const int* skip, cudaStream_t st)
+{
+    auto go = [&](auto launch) { launch(nn, Mr, N, K, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip, st); };
+    if (N == 1) go(launch_mv<1, MT>);
+    else if (N == 2) go(launch_mv<2, MT>);
+    else if (N <= 4) go(launch_mv<4, MT>);
+    else go(launch_mv<8, MT>);
 }
 
 // O = [acc] O + alpha A B over the merges of a level (B [K][N], O [M][N]):
@@ -435,8 +470,7 @@ void if_product(int nn, int Mr, int N, int K, const MT* A, long long lda, long l
         return;
     }
     hps::prof_begin(hps::KC_MISC, st);
-    if (N <= 2) launch_mv<2, MT>(nn, Mr, N, K, A, lda, sA, B, sB, N, 1, O, sO, N, 1, alpha, acc ? 1 : 0, skip, st);
-    else launch_mv<8, MT>(nn, Mr, N, K, A, lda, sA, B, sB, N, 1, O, sO, N, 1, alpha, acc ? 1 : 0, skip, st);
+    launch_mv_n<MT>(nn, Mr, N, K, A, lda, sA, B, sB, N, 1, O, sO, N, 1, alpha, acc ? 1 : 0, skip, st);
     hps::prof_end(hps::KC_MISC, st, 2.0 * nn * Mr * (double)N * K,
                   (double)nn * ((double)Mr * K * sizeof(MT) + 8.0 * (double)Mr * N));
 }
@@ -556,7 +590,15 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     // FP64 refinement recovers the digits
     const bool tc = sizeof(MT) == 4 && s >= 256;
     hps::Plan PL = hps::make_plan(s, e + s, tc ? HPS_BF16_IR : prec, 0, tc, false);
-    const size_t need = PL.per_box * (size_t)L.nn;
+    // The merged maps' products E S in FP32: with 3 x BF16 operands (FP32's 24
+    // bits, FP32 accumulation) on the tensor cores where the map's rows are
+    // 16-byte aligned (e a multiple of 4: every even q), on the CUDA cores
+    // elsewhere.  8 x 8 x 8 boxes at p = 12: 145 ms on the CUDA cores, 17 ms with
+    // the operand packs.
+    const bool tc_merge = sizeof(MT) == 4 && e > 0 && e % 4 == 0;
+    const size_t lu_bytes = PL.per_box * (size_t)L.nn;
+    const size_t merge_bytes = tc_merge ? hps::tc_gemm_f32_scratch(e, e, s) * (size_t)L.nn : 0;
+    const size_t need = hps::align_up(lu_bytes, 1024) + merge_bytes;
     if (need > *ws_bytes) {
         if (*ws) { cudaStreamSynchronize(st); cudaFree(*ws); *ws = nullptr; *ws_bytes = 0; }
         if (cudaMalloc(ws, need) != cudaSuccess) { cudaGetLastError(); return HPS_ENOMEM; }
@@ -591,7 +633,16 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     k_if_extract<MT><<<dim3((unsigned)s, (unsigned)L.nn), 256, 0, st>>>(w.M, PL.ldm, w.sM, s, e,
                                                                          static_cast<MT*>(L.S),
                                                                          static_cast<MT*>(L.Winv));
-    if (e > 0)
+    if constexpr (sizeof(MT) == 4) {
+        if (tc_merge) {   // Tn -= E X with X = -S, the solved columns of M
+            if (!tc_done) hps::tc_reset_abort(st);
+            if (!hps::tc_gemm_f32(e, e, s, static_cast<const float*>(L.E), s, (long long)e * s, w.M + s, PL.ldm, w.sM,
+                                  static_cast<float*>(L.Tn), e, (long long)e * e, *d_status, L.nn,
+                                  static_cast<char*>(*ws) + hps::align_up(lu_bytes, 1024), st))
+                return HPS_ECUDA;
+        }
+    }
+    if (e > 0 && !tc_merge)
         if_merge_product<MT>(L.nn, e, s, static_cast<const MT*>(L.E), static_cast<const MT*>(L.S),
                              static_cast<MT*>(L.Tn), st);
     if (cudaGetLastError() != cudaSuccess) return HPS_ECUDA;
@@ -849,12 +900,8 @@ hps_status hps_interface_solve(hps_interface* F, int nrhs, const double* h, cons
             return HPS_ECUDA;
         // hcur[box][c][r] += sum_j T[box][r][j] ub[box][c][j]
         hps::prof_begin(hps::KC_MISC, st);
-        if (R <= 2)
-            launch_mv<2, double>(F->nbox, m, R, m, F->Tcopy, m, (long long)m * m, ub, (long long)R * m, 1, m, F->hcur,
-                                 (long long)R * m, 1, m, 1.0, 1, F->rflag, st);
-        else
-            launch_mv<8, double>(F->nbox, m, R, m, F->Tcopy, m, (long long)m * m, ub, (long long)R * m, 1, m, F->hcur,
-                                 (long long)R * m, 1, m, 1.0, 1, F->rflag, st);
+        launch_mv_n<double>(F->nbox, m, R, m, F->Tcopy, m, (long long)m * m, ub, (long long)R * m, 1, m, F->hcur,
+                            (long long)R * m, 1, m, 1.0, 1, F->rflag, st);
         hps::prof_end(hps::KC_MISC, st, 2.0 * F->nbox * (double)m * m * R, 8.0 * F->nbox * (double)m * m);
         solve_sweeps<float>(F, R, F->hcur, nullptr, F->du, F->rflag, st);
         k_if_update<<<(unsigned)std::min<long long>((total + 255) / 256, 4096), 256, 0, st>>>(total, F->du, ub,
