@@ -9,7 +9,8 @@
 //   1. load the block; for each earlier block: the rows that were its pivots
 //      hand their entries over, the block's unit triangle (its inverse, kept)
 //      turns them into rows of U, and every other row subtracts its stored
-//      multipliers times them (16 multiply-adds per value read back);
+//      multipliers times them (16 multiply-adds per value read back; FP64 as
+//      digit products on the tensor cores, see hps_digits.cuh);
 //   2. factor the block: per column every warp offers its largest candidate
 //      with its row, the CTA picks one after one barrier (in a cluster the
 //      CTAs' offers are exchanged through distributed shared memory and a
@@ -18,8 +19,8 @@
 //   3. multipliers of the rows still active go to a scratch block by columns,
 //      where a warp reads and writes whole lines.
 // At the end every row goes to its place in the matrix: pivot rows on top, rows
-// they displaced where the row swaps would have taken them; perm[r] is the old
-// row at position r.
+// they displaced to the places that they left; perm[r] is the old row at
+// position r.
 //
 // What bounds it: with many boxes the multiply-adds of the elimination
 // (R nb^2 / 2 per box: the FP32 pipes at 128 a clock, the FP64 pipes at 2);
@@ -31,6 +32,7 @@
 #include <climits>
 #include <type_traits>
 
+#include "hps_digits.cuh"
 #include "hps_internal.h"
 #include "hps_ptx.cuh"
 
@@ -122,6 +124,34 @@ __device__ __forceinline__ bool warp_argmax(unsigned long long& key, int& row)
     return mine;
 }
 
+// Index of the best of eight offers (keys and rows on 16 bytes), with its key
+// and row: a tree of comparisons, the reduction instructions' latency saved.
+template <typename K>
+__device__ __forceinline__ int best_offer(const K* ks, const int* rs, K& key, int& row)
+{
+    K k[8];
+    int r[8], id[8];
+#pragma unroll
+    for (int i = 0; i < 8 * (int)sizeof(K) / 16; ++i)
+        *reinterpret_cast<uint4*>(&k[i * 16 / (int)sizeof(K)]) = reinterpret_cast<const uint4*>(ks)[i];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) *reinterpret_cast<int4*>(&r[4 * i]) = reinterpret_cast<const int4*>(rs)[i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) id[i] = i;
+#pragma unroll
+    for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+        for (int i = 0; i < h; ++i)
+            if (k[i + h] > k[i] || (k[i + h] == k[i] && r[i + h] < r[i])) {
+                k[i] = k[i + h];
+                r[i] = r[i + h];
+                id[i] = id[i + h];
+            }
+    key = k[0];
+    row = r[0];
+    return id[0];
+}
+
 // 1 / x.  FP64: on the integer pipe (a division is ten dependent operations of
 // 64 clocks a warp on the FP64 pipe): y, 1 / m to 22 bits from FP32, then
 // y (1 + e + e^2) with e = 1 - m y in fixed point, |e|^3 below 2^-66, rounded
@@ -201,6 +231,21 @@ __device__ __forceinline__ float4* tile_unit(T* tile, int r, int q)
     return reinterpret_cast<float4*>(tile) + r * 4 + (q ^ ((r >> 1) & 3));
 }
 
+// The same for rows of 128 bytes (16 FP64 values).
+__device__ __forceinline__ double2* tile_unit128(double* tile, int r, int q)
+{
+    return reinterpret_cast<double2*>(tile) + r * 8 + (q ^ (r & 7));
+}
+
+// D += A B, m16n8k16, FP16 in, FP32 accumulate.
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
+}
+
 template <typename T>
 struct PanelArgs {
     T* M;
@@ -217,23 +262,31 @@ struct PanelArgs {
 // Shared memory of a panel CTA.
 template <typename T, int IB>
 struct PanelSmem {
-    alignas(16) T tile[PW][32 * 64 / sizeof(T)];   // per warp: 32 rows of 64 bytes between row and column order
+    // per warp: 32 rows of 64 bytes between row and column order (FP64: of IB values, for its products)
+    alignas(16) T tile[PW][sizeof(T) == 8 ? 32 * IB : 512];
     alignas(16) T inv[kMaxNB / IB][IB][IB];        // inverses of the blocks' unit lower triangles
     alignas(16) T raw[2][IB][IB], u[IB][IB];       // a block's pivot rows before (alternating: a CTA may run one
                                                    // block ahead of its cluster) and after its triangle
+    alignas(16) uint2 ud[sizeof(T) == 8 ? IB / 8 : 1][DG_S][32];   // FP64: u's digits as MMA operands
+    int ue[IB];                                    // and the scales of its columns
     alignas(16) T cand[2][PW][IB];                 // the warps' offers
     alignas(16) T offer[2][kMaxCluster][IB];       // the CTAs' offers
-    PivotKey<T> ckey[2][PW], okey[2][kMaxCluster];
-    int crow[2][PW], orow[2][kMaxCluster];
+    T crcp[2][PW], orcp[2][kMaxCluster];           // reciprocals of the offered pivots
+    alignas(16) PivotKey<T> ckey[2][PW];
+    alignas(16) PivotKey<T> okey[2][kMaxCluster];
+    alignas(16) int crow[2][PW];
+    alignas(16) int orow[2][kMaxCluster];
     int prow[kMaxNB];                              // row chosen for each column
-    int pp[kMaxNB];                                // position it had been swapped to
+    int vac[kMaxNB], dest[kMaxNB];                 // places left by pivots below the top; where displaced rows go
+    int nd[4], nv[4];
     unsigned char is_pivot[kMaxNB];
     int sing;
 };
+static_assert(PW == 8 && kMaxCluster == 8, "best_offer compares eight");
 
-// CTAs per SM: two of FP32 (77 KiB of shared memory at nb = 128), three of FP64 where a row is 32 registers.
+// CTAs per SM by the registers of a thread's rows: two of up to 64 (FP32) or 32 (FP64, whose products take 90 more).
 template <typename T>
-constexpr int panel_min_blocks(int regs) { return regs <= 32 && sizeof(T) == 8 ? 3 : regs <= 64 ? 2 : 1; }
+constexpr int panel_min_blocks(int regs) { return regs <= (sizeof(T) == 4 ? 64 : 32) ? 2 : 1; }
 
 template <typename T, int RPT, int IB>
 __global__ void __launch_bounds__(PT, panel_min_blocks<T>(RPT * IB * (int)sizeof(T) / 4))
@@ -259,10 +312,15 @@ k_panel(const PanelArgs<T> a)
     for (int rr = 0; rr < RPT; ++rr) pidx[rr] = row_of(rr) < R0 ? -1 : -2;
     if (tid < kMaxNB) s.is_pivot[tid] = 0;
     if (tid == 0) s.sing = 0;
+    if (tid < 2 * kMaxCluster) (&s.okey[0][0])[tid] = 0;
     if (C > 1) cluster_sync();   // every CTA of the cluster runs before its shared memory is written
 
     constexpr int CU = 16 / sizeof(T), CW = 4 * CU;   // entries of a 16-byte unit and of a 64-byte row piece
     T* tile = s.tile[warp];
+    auto tile_row = [](T* t, int r, int q) {   // FP64 product rows: IB values each
+        if constexpr (IB == 16) return tile_unit128(reinterpret_cast<double*>(t), r, q);
+        else return reinterpret_cast<double2*>(tile_unit(t, r, q));
+    };
     T* Lt = a.Lt + box * a.sL;
     T x[RPT][IB];
     for (int b = 0; b < nblk; ++b) {
@@ -306,7 +364,8 @@ k_panel(const PanelArgs<T> a)
         }
         for (int e = 0; e < b; ++e) {
             const int je = e * IB;
-            constexpr int JC = RPT * (int)sizeof(T) >= 32 ? 2 : 4;   // multipliers read ahead per row
+            // FP32: multipliers read ahead per row, the first ones before the barrier
+            constexpr int JC = sizeof(T) == 8 ? 1 : 16 / RPT;
             T l[RPT][JC];
             auto load_l = [&](int j0) {
 #pragma unroll
@@ -316,7 +375,7 @@ k_panel(const PanelArgs<T> a)
                     for (int j = 0; j < JC; ++j) l[rr][j] = on ? Lt[(long long)(je + j0 + j) * R0 + row_of(rr)] : T(0);
                 }
             };
-            load_l(0);
+            if constexpr (sizeof(T) == 4) load_l(0);
 #pragma unroll
             for (int rr = 0; rr < RPT; ++rr)
                 if (pidx[rr] >= je && pidx[rr] < je + IB) {
@@ -343,21 +402,125 @@ k_panel(const PanelArgs<T> a)
                 LU[(je + i) * ldl + jb + c] = v;
             }
             __syncthreads();
+            if constexpr (sizeof(T) == 4) {
 #pragma unroll 1
-            for (int j0 = 0; j0 < IB; j0 += JC) {
-                T lc[RPT][JC];
-#pragma unroll
-                for (int rr = 0; rr < RPT; ++rr)
-#pragma unroll
-                    for (int j = 0; j < JC; ++j) lc[rr][j] = l[rr][j];
-                if (j0 + JC < IB) load_l(j0 + JC);
-#pragma unroll
-                for (int j = 0; j < JC; ++j) {
-                    T uv[IB];
-                    load_row<T, IB>(uv, s.u[j0 + j]);
+                for (int j0 = 0; j0 < IB; j0 += JC) {
+                    T lc[RPT][JC];
 #pragma unroll
                     for (int rr = 0; rr < RPT; ++rr)
-                        if (rr < nrr) sub_row(x[rr], lc[rr][j], uv);
+#pragma unroll
+                        for (int j = 0; j < JC; ++j) lc[rr][j] = l[rr][j];
+                    if (j0 + JC < IB) load_l(j0 + JC);
+#pragma unroll
+                    for (int j = 0; j < JC; ++j) {
+                        T uv[IB];
+                        load_row<T, IB>(uv, s.u[j0 + j]);
+#pragma unroll
+                        for (int rr = 0; rr < RPT; ++rr)
+                            if (rr < nrr) sub_row(x[rr], lc[rr][j], uv);
+                    }
+                }
+            } else {
+                // FP64: the product of the multipliers with u from exact digits
+                // (K = IB <= 16: every accumulator stays below 2^21); as 16 multiply-adds
+                // per entry on the FP64 pipe, 64 clocks a warp each, it took seven times as long
+                const int g = lane >> 2, q = lane & 3;
+                if (warp < IB / 8) {
+                    double v[4];
+                    int ex = E_MIN;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const int kk = 2 * q + (t & 1) + 8 * (t >> 1);
+                        v[t] = kk < IB ? s.u[kk < IB ? kk : 0][8 * warp + g] : 0.0;
+                        ex = max(ex, exp_of(v[t]));
+                    }
+                    ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 1));
+                    ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 2));
+                    uint32_t d[DG_S][2];
+                    split4(v, ex, d);
+#pragma unroll
+                    for (int t = 0; t < DG_S; ++t) s.ud[warp][t][lane] = make_uint2(d[t][0], d[t][1]);
+                    if (q == 0) s.ue[8 * warp + g] = ex == E_BAD ? E_NAN : ex - 1018;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int rr = 0; rr < RPT; ++rr) {
+                    if (rr >= nrr) continue;
+                    const bool mineon = pidx[rr] == -1 || pidx[rr] >= je + IB;
+                    const uint32_t onm = __ballot_sync(0xffffffffu, mineon);
+                    const int row0 = row_of(rr) - lane;
+#pragma unroll 1
+                    for (int mt = 0; mt < 2; ++mt) {
+                        uint32_t ad[2][DG_S][2];
+                        int ea[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int rl = 16 * mt + 8 * h + g;
+                            const bool on = onm >> rl & 1;
+                            double v[4];
+                            int ex = E_MIN;
+#pragma unroll
+                            for (int t = 0; t < 4; ++t) {
+                                const int kk = 2 * q + (t & 1) + 8 * (t >> 1);
+                                v[t] = on && kk < IB ? Lt[(long long)(je + kk) * R0 + row0 + rl] : 0.0;
+                                ex = max(ex, exp_of(v[t]));
+                            }
+                            ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 1));
+                            ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 2));
+                            split4(v, ex, ad[h]);
+                            ea[h] = ex == E_BAD ? E_NAN : ex;
+                        }
+#pragma unroll 1
+                        for (int nt = 0; nt < IB / 8; ++nt) {
+                            uint2 bd[DG_S];
+#pragma unroll
+                            for (int t = 0; t < DG_S; ++t) bd[t] = s.ud[nt][t][lane];
+                            // accumulators two at a time, joined as they are done
+                            long long V[4] = {0, 0, 0, 0};
+#pragma unroll
+                            for (int t = 0; t < DG_S; t += 2) {
+                                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                                for (int i = 0; i <= t; ++i)
+                                    mma16816(c0, ad[0][i][0], ad[1][i][0], ad[0][i][1], ad[1][i][1], bd[t - i]);
+#pragma unroll
+                                for (int i = 0; i <= t + 1; ++i)
+                                    mma16816(c1, ad[0][i][0], ad[1][i][0], ad[0][i][1], ad[1][i][1], bd[t + 1 - i]);
+                                constexpr float MG = 12582912.0f;
+                                constexpr uint32_t MB = 0x4B400000u;
+#pragma unroll
+                                for (int o = 0; o < 4; ++o) {
+                                    const int w2 = (int)(__float_as_uint(__fadd_rn(c0[o], MG)) * 256u +
+                                                         (__float_as_uint(__fadd_rn(c1[o], MG)) - MB * 257u));
+                                    if (t == 0) V[o] = (long long)((uint64_t)(uint32_t)(w2 << 7) << 32);
+                                    else if (t == 2) V[o] += (long long)w2 * (1 << 23);
+                                    else if (t == 4) V[o] += (long long)w2 * 128;
+                                    else V[o] += (w2 + 256) >> 9;
+                                }
+                            }
+                            const int2 ue = *reinterpret_cast<const int2*>(&s.ue[8 * nt + 2 * q]);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                int eb0, eb1;
+                                double2 r;
+                                r.x = round_fixed(V[2 * h], ea[h] + ue.x, eb0);
+                                r.y = round_fixed(V[2 * h + 1], ea[h] + ue.y, eb1);
+                                if ((unsigned)eb0 > 2045u) r.x = finish_odd(r.x, ea[h] + ue.x, eb0);
+                                if ((unsigned)eb1 > 2045u) r.y = finish_odd(r.y, ea[h] + ue.y, eb1);
+                                *tile_row(tile, 16 * mt + 8 * h + g, 4 * nt + q) = r;
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if (mineon) {
+#pragma unroll
+                        for (int c = 0; c < IB / 2; ++c) {
+                            const double2 r = *tile_row(tile, lane, c);
+                            x[rr][2 * c] -= r.x;
+                            x[rr][2 * c + 1] -= r.y;
+                        }
+                    }
+                    __syncwarp();
                 }
             }
         }
@@ -365,28 +528,40 @@ k_panel(const PanelArgs<T> a)
         // column, so that the column at hand is always x[.][0] and the loop stays
         // small (unrolled over the columns it outgrows the instruction cache);
         // the multipliers fill the registers that come free at the end.
-#pragma unroll 1
-        for (int c = 0; c < w; ++c) {
-            const int cur = c & 1;
-            PivotKey<T> key = 0;
-            int row = INT_MAX, brr = 0;
+        PivotKey<T> key;
+        int row, brr;
+        T rcp;
+        bool mine;
+        // the warp's offer for the column in x[.][0], with the reciprocal that its
+        // elimination will need taken while the reductions run
+        auto offer = [&]() {
+            key = 0;
+            row = INT_MAX;
+            brr = 0;
+            T xb = T(1);
 #pragma unroll
             for (int rr = 0; rr < RPT; ++rr) {
                 const PivotKey<T> kk = pidx[rr] == -1 ? pivot_key(x[rr][0]) : PivotKey<T>(0);
-                if (kk > key) { key = kk; row = row_of(rr); brr = rr; }
+                if (kk > key) { key = kk; row = row_of(rr); brr = rr; xb = x[rr][0]; }
             }
-            if (warp_argmax(key, row)) {
+            rcp = reciprocal(xb == T(0) ? T(1) : xb);   // a zero pivot: recorded below, the arithmetic stays finite
+            mine = warp_argmax(key, row);
+        };
+        offer();
+#pragma unroll 1
+        for (int c = 0; c < w; ++c) {
+            const int cur = c & 1;
+            if (mine) {
 #pragma unroll
                 for (int rr = 0; rr < RPT; ++rr)
                     if (rr == brr) store_row<T, IB>(s.cand[cur][warp], x[rr]);
+                s.crcp[cur][warp] = rcp;
             }
             if (lane == 0) { s.ckey[cur][warp] = key; s.crow[cur][warp] = row; }
             __syncthreads();
-            // the CTA's best (every warp finds it for itself)
-            key = lane < PW ? s.ckey[cur][lane] : PivotKey<T>(0);
-            row = lane < PW ? s.crow[cur][lane] : INT_MAX;
-            unsigned who = __ballot_sync(0xffffffffu, warp_argmax(key, row));
-            const T* pv = s.cand[cur][who ? __ffs((int)who) - 1 : 0];
+            int best = best_offer(s.ckey[cur], s.crow[cur], key, row);
+            const T* pv = s.cand[cur][best];
+            T rinv = s.crcp[cur][best];
             if (C > 1) {
                 if (warp == 0) {
                     for (int e = lane; e < C * IB; e += 32) {
@@ -396,27 +571,19 @@ k_panel(const PanelArgs<T> a)
                     if (lane < C) {
                         remote_store(remote_addr(&s.okey[cur][rank], (unsigned)lane), key);
                         remote_store(remote_addr(&s.orow[cur][rank], (unsigned)lane), row);
+                        remote_store(remote_addr(&s.orcp[cur][rank], (unsigned)lane), rinv);
                     }
                 }
                 cluster_sync();
-                key = lane < C ? s.okey[cur][lane] : PivotKey<T>(0);
-                row = lane < C ? s.orow[cur][lane] : INT_MAX;
-                who = __ballot_sync(0xffffffffu, warp_argmax(key, row));
-                pv = s.offer[cur][who ? __ffs((int)who) - 1 : 0];
+                best = best_offer(s.okey[cur], s.orow[cur], key, row);
+                pv = s.offer[cur][best];
+                rinv = s.orcp[cur][best];
             }
-            T piv = pv[0];
-            if (piv == T(0)) {   // exactly singular: record it and keep the arithmetic finite
-                if (tid == 0) s.sing = 1;
-                piv = T(1);
-            }
-            const T rinv = reciprocal(piv);
             if (tid < IB) LU[(jb + c) * ldl + jb + ((tid + c) & (IB - 1))] = pv[tid];
             if (tid == 32) {
                 s.prow[jb + c] = row;
                 if (row < nb) s.is_pivot[row] = 1;
-                int pos = row;   // follow the swaps that moved the row before
-                while (pos < jb + c) pos = s.pp[pos];
-                s.pp[jb + c] = pos;
+                if (key == 2) s.sing = 1;   // |pivot| = 0
             }
             T l[RPT];
 #pragma unroll
@@ -442,6 +609,7 @@ k_panel(const PanelArgs<T> a)
                             if constexpr (sizeof(T) == 4) x[rr][i - 1] = x[rr][i] - l[rr] * pu;
                             else x[rr][i - 1] = col ? x[rr][i] - l[rr] * pu : x[rr][i];
                         }
+                    if (i == 1) offer();   // the next column is known first; its reductions overlap the rest
                 }
             }
 #pragma unroll
@@ -484,8 +652,21 @@ k_panel(const PanelArgs<T> a)
     else __syncthreads();
 
     // Every row that became no pivot goes to its place: below the panel's top
-    // it stays, and one that a pivot displaced from the top moved to where that
-    // pivot had been, on from there if a later column took that place too.
+    // it stays; the i-th row that pivots displaced from the top takes the i-th
+    // place that they left below it.
+    {
+        const bool disp = tid < nb && !s.is_pivot[tid < nb ? tid : 0], left = tid < nb && s.prow[tid < nb ? tid : 0] >= nb;
+        const uint32_t md = __ballot_sync(0xffffffffu, disp), mv = __ballot_sync(0xffffffffu, left);
+        const uint32_t below = (1u << lane) - 1;
+        if (lane == 0 && warp < 4) { s.nd[warp] = __popc(md); s.nv[warp] = __popc(mv); }
+        __syncthreads();
+        int od = __popc(md & below), ov = __popc(mv & below);
+        for (int q = 0; q < warp && q < 4; ++q) { od += s.nd[q]; ov += s.nv[q]; }
+        if (left) s.vac[ov] = s.prow[tid];
+        __syncthreads();
+        if (disp) s.dest[tid] = s.vac[od];
+        __syncthreads();
+    }
     int* pb = a.perm + box * a.sP;
     for (int rr = 0; rr < nrr; ++rr) {
         const int row = row_of(rr);
@@ -498,8 +679,7 @@ k_panel(const PanelArgs<T> a)
                     if (q == rr) pivot = pidx[q] >= 0;
             }
             if (!pivot) {
-                pos = row;
-                while (pos < nb) pos = s.pp[pos];
+                pos = row < nb ? s.dest[row] : row;
                 pb[pos] = row;
             }
         }
@@ -585,31 +765,45 @@ __device__ void tri_inverse(T* A, T* X, int P, bool lower, int tid)
         for (int i = 0; i < 16; ++i) X[(q0 + i) * P + q0 + c] = y[i];
     }
     __syncthreads();
+    // V neighbouring columns per item: one 16-byte read and one broadcast per V
+    // multiply-adds (X is zero on the far side of its diagonal, so a loop may
+    // start or end at the item's first or last column)
+    constexpr int V = 16 / sizeof(T);
     for (int b = 16; b < P; b *= 2) {
-        const int items = (P / (2 * b)) * b * b;
+        const int items = (P / (2 * b)) * b * (b / V);
         // middle products into the free triangle of A
         for (int it = tid; it < items; it += TI) {
-            const int pr = it / (b * b), e = it - pr * b * b, r = e / b, c = e - r * b, i0 = 2 * b * pr;
-            T acc = T(0);
-            if (lower) {   // C A1^{-1}: C = A[i0+b+r][i0+t], A1^{-1} lower
-                for (int t = c; t < b; ++t) acc += A[(i0 + b + r) * P + i0 + t] * X[(i0 + t) * P + i0 + c];
-                A[(i0 + r) * P + i0 + b + c] = acc;
-            } else {       // B D^{-1}: B = A[i0+r][i0+b+t], D^{-1} upper
-                for (int t = 0; t <= c; ++t) acc += A[(i0 + r) * P + i0 + b + t] * X[(i0 + b + t) * P + i0 + b + c];
-                A[(i0 + b + r) * P + i0 + c] = acc;
+            const int pr = it / (b * (b / V)), e = it - pr * (b * (b / V)), r = e / (b / V), c = (e - r * (b / V)) * V,
+                      i0 = 2 * b * pr;
+            T acc[V] = {};
+            const T* m = lower ? A + (i0 + b + r) * P + i0 : A + (i0 + r) * P + i0 + b;
+            const T* xr = lower ? X + i0 * P + i0 + c : X + (i0 + b) * P + i0 + b + c;
+            const int t0 = lower ? c : 0, t1 = lower ? b : c + V;   // C A1^{-1} (A1^{-1} lower) or B D^{-1} (upper)
+#pragma unroll 4
+            for (int t = t0; t < t1; ++t) {
+                T xv[V];
+                load_row<T, V>(xv, xr + t * P);
+#pragma unroll
+                for (int q = 0; q < V; ++q) acc[q] += m[t] * xv[q];
             }
+            store_row<T, V>(lower ? A + (i0 + r) * P + i0 + b + c : A + (i0 + b + r) * P + i0 + c, acc);
         }
         __syncthreads();
         for (int it = tid; it < items; it += TI) {
-            const int pr = it / (b * b), e = it - pr * b * b, r = e / b, c = e - r * b, i0 = 2 * b * pr;
-            T acc = T(0);
-            if (lower) {   // -D^{-1} (C A1^{-1}), D^{-1} lower
-                for (int t = 0; t <= r; ++t) acc -= X[(i0 + b + r) * P + i0 + b + t] * A[(i0 + t) * P + i0 + b + c];
-                X[(i0 + b + r) * P + i0 + c] = acc;
-            } else {       // -A1^{-1} (B D^{-1}), A1^{-1} upper
-                for (int t = r; t < b; ++t) acc -= X[(i0 + r) * P + i0 + t] * A[(i0 + b + t) * P + i0 + c];
-                X[(i0 + r) * P + i0 + b + c] = acc;
+            const int pr = it / (b * (b / V)), e = it - pr * (b * (b / V)), r = e / (b / V), c = (e - r * (b / V)) * V,
+                      i0 = 2 * b * pr;
+            T acc[V] = {};
+            const T* m = lower ? X + (i0 + b + r) * P + i0 + b : X + (i0 + r) * P + i0;
+            const T* xr = lower ? A + i0 * P + i0 + b + c : A + (i0 + b) * P + i0 + c;
+            const int t0 = lower ? 0 : r, t1 = lower ? r + 1 : b;   // -D^{-1} (..), D^{-1} lower, or -A1^{-1} (..), upper
+#pragma unroll 4
+            for (int t = t0; t < t1; ++t) {
+                T xv[V];
+                load_row<T, V>(xv, xr + t * P);
+#pragma unroll
+                for (int q = 0; q < V; ++q) acc[q] -= m[t] * xv[q];
             }
+            store_row<T, V>(lower ? X + (i0 + b + r) * P + i0 + c : X + (i0 + r) * P + i0 + b + c, acc);
         }
         __syncthreads();
     }
@@ -631,6 +825,7 @@ k_tri_inv(const T* __restrict__ M, long long ldm, long long sM, int k, int nb, T
     T* A = reinterpret_cast<T*>(smem_raw);   // Pd x Pd, padded with the identity
     T* X = A + Pd * Pd;
     const T* D = M + box * sM + (long long)k * ldm + k;
+#pragma unroll 8
     for (int idx = tid; idx < Pd * Pd; idx += TI) {
         const int r = idx / Pd, c = idx - r * Pd;
         const bool in = r < nb && c < nb && (lower ? c < r : c >= r);
@@ -681,7 +876,7 @@ template <typename T>
 PanelShape panel_shape(int i)
 {
     static const PanelShape f[4] = {{1, 16, 2}, {2, 16, 2}, {4, 16, 2}, {8, 16, 1}};
-    static const PanelShape d[4] = {{1, 16, 3}, {2, 16, 2}, {4, 16, 1}, {8, 8, 1}};
+    static const PanelShape d[4] = {{1, 16, 2}, {2, 16, 1}, {4, 16, 1}, {8, 8, 1}};
     return sizeof(T) == 4 ? f[i] : d[i];
 }
 template <typename T>
