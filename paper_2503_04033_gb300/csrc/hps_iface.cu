@@ -392,7 +392,8 @@ __global__ void __launch_bounds__(256) k_if_mv(int Mr, int K, int N, int KS, con
                         if constexpr (sizeof(MT) == 4) a = hps::f2d(av[r][u]);
                         else a = av[r][u];
 #pragma unroll
-                        for (int c = 0; c < NC; ++c) s[r][c] += a * bv[u][c];
+                        for (int c = 0; c < NC; ++c)
+                            if (c0 + c < N) s[r][c] += a * bv[u][c];
                     }
             }
         }
@@ -592,10 +593,11 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     hps::Plan PL = hps::make_plan(s, e + s, tc ? HPS_BF16_IR : prec, 0, tc, false);
     // The merged maps' products E S in FP32: with 3 x BF16 operands (FP32's 24
     // bits, FP32 accumulation) on the tensor cores where the map's rows are
-    // 16-byte aligned (e a multiple of 4: every even q), on the CUDA cores
-    // elsewhere.  8 x 8 x 8 boxes at p = 12: 145 ms on the CUDA cores, 17 ms with
+    // 16-byte aligned (e a multiple of 4: every even q) and the product pays for
+    // its two packs (1e8 multiply-adds take the CUDA cores 12 us), on the CUDA
+    // cores elsewhere.  8 x 8 x 8 boxes at p = 12: 145 ms on the CUDA cores, 17 ms with
     // the operand packs.
-    const bool tc_merge = sizeof(MT) == 4 && e > 0 && e % 4 == 0;
+    const bool tc_merge = sizeof(MT) == 4 && e > 0 && e % 4 == 0 && (double)L.nn * e * e * s >= 1e8;
     const size_t lu_bytes = PL.per_box * (size_t)L.nn;
     const size_t merge_bytes = tc_merge ? hps::tc_gemm_f32_scratch(e, e, s) * (size_t)L.nn : 0;
     const size_t need = hps::align_up(lu_bytes, 1024) + merge_bytes;
