@@ -422,19 +422,22 @@ __device__ __forceinline__ void block_sum_add(V v, double* out)
 
 // X = src in FP64 (the first solution of the refinement); with xnorm, also
 // ||X||^2 per box into xnorm[2 box + 1] (FP32 partial sums: the stopping rule
-// needs the size of X, not its digits).  CTAs loop over rows, threads over
-// columns.
+// needs the size of X, not its digits).  CTAs loop over rows, 2^lg threads over
+// the columns of each: with a whole CTA per row one column of 64 boxes at n =
+// 1000 took 41 us, a thread in 256 at work.
 template <typename TS>
 __global__ void __launch_bounds__(256)
 k_extract(const TS* __restrict__ src, long long lds, long long sS, int n, int ncols, double* __restrict__ X,
-          long long ldx, long long sX, double* xnorm)
+          long long ldx, long long sX, double* xnorm, int lg)
 {
     const int box = blockIdx.y;
     float xn = 0.0f;
-    for (int r = blockIdx.x; r < n; r += gridDim.x) {
+    const int c0 = threadIdx.x & ((1 << lg) - 1), rg = blockDim.x >> lg;
+#pragma unroll 4
+    for (int r = blockIdx.x * rg + (threadIdx.x >> lg); r < n; r += gridDim.x * rg) {
         const TS* srow = src + box * sS + (long long)r * lds;
         double* xrow = X + box * sX + (long long)r * ldx;
-        for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
+        for (int c = c0; c < ncols; c += 1 << lg) {
             const TS v = srow[c];
             if constexpr (sizeof(TS) == 4) xrow[c] = f2d(v);
             else xrow[c] = double(v);
@@ -974,16 +977,18 @@ k_residual_df(int p, int n, const float4* __restrict__ DF, const float2* __restr
 // after the update, in FP64, to norms[2 box + 1].
 __global__ void __launch_bounds__(256)
 k_ir_update(const float* __restrict__ D, long long ldd, long long sD, int n, int ncols, double* __restrict__ X,
-            long long ldx, long long sX, double* norms, const int* skip, int want_xn)
+            long long ldx, long long sX, double* norms, const int* skip, int want_xn, int lg)
 {
     const int box = blockIdx.y;
     if (skip && skip[box]) return;
     float dn = 0.0f;
     double xn = 0.0;
-    for (int r = blockIdx.x; r < n; r += gridDim.x) {
+    const int c0 = threadIdx.x & ((1 << lg) - 1), rg = blockDim.x >> lg;   // columns and rows as in k_extract
+#pragma unroll 4
+    for (int r = blockIdx.x * rg + (threadIdx.x >> lg); r < n; r += gridDim.x * rg) {
         const float* drow = D + box * sD + (long long)r * ldd;
         double* xrow = X + box * sX + (long long)r * ldx;
-        for (int c = threadIdx.x; c < ncols; c += blockDim.x) {
+        for (int c = c0; c < ncols; c += 1 << lg) {
             const float d = drow[c];
             const double x = xrow[c] + f2d(d);
             xrow[c] = x;
@@ -1307,13 +1312,22 @@ void launch_dn(const Geometry& g, int nbox, const double* X, long long ldx, long
     prof_end(KC_DN, st, 2.0 * nbox * g.m * (double)ncols * g.q, (double)nbox * ((double)g.n + g.m) * ncols * 8);
 }
 
+// log2 of the threads of a 256-thread CTA that share a row of ncols columns.
+static int column_threads_lg(int ncols)
+{
+    int lg = 0;
+    while (lg < 8 && (1 << lg) < ncols) ++lg;
+    return lg;
+}
+
 template <typename TS>
 void launch_extract(const TS* src, long long lds, long long sS, int n, int ncols,
                     double* X, long long ldx, long long sX, int nbox, cudaStream_t st, double* xnorm)
 {
-    dim3 grd((unsigned)std::min(n, 96), (unsigned)nbox);
+    const int lg = column_threads_lg(ncols);
+    dim3 grd((unsigned)std::min((n + (256 >> lg) - 1) / (256 >> lg), 96), (unsigned)nbox);
     prof_begin(KC_REFINE, st);
-    k_extract<TS><<<grd, 256, 0, st>>>(src, lds, sS, n, ncols, X, ldx, sX, xnorm);
+    k_extract<TS><<<grd, 256, 0, st>>>(src, lds, sS, n, ncols, X, ldx, sX, xnorm, lg);
     prof_end(KC_REFINE, st, 0.0, (double)nbox * n * (double)ncols * (sizeof(TS) + 8));
 }
 
@@ -1494,9 +1508,10 @@ void launch_ir_update(const float* D, long long ldd, long long sD, int n, int nc
                       double* X, long long ldx, long long sX, double* norms,
                       const int* skip, int nbox, cudaStream_t st, bool want_xn)
 {
-    dim3 grd((unsigned)std::min(n, 96), (unsigned)nbox);
+    const int lg = column_threads_lg(ncols);
+    dim3 grd((unsigned)std::min((n + (256 >> lg) - 1) / (256 >> lg), 96), (unsigned)nbox);
     prof_begin(KC_REFINE, st);
-    k_ir_update<<<grd, 256, 0, st>>>(D, ldd, sD, n, ncols, X, ldx, sX, norms, skip, want_xn ? 1 : 0);
+    k_ir_update<<<grd, 256, 0, st>>>(D, ldd, sD, n, ncols, X, ldx, sX, norms, skip, want_xn ? 1 : 0, lg);
     prof_end(KC_REFINE, st, 0.0, (double)nbox * n * (double)ncols * 20.0);
 }
 
