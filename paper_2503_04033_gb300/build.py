@@ -18,7 +18,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libhps.so")
 BUILD_DIR = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["hps_abi.cu", "hps_lu.cu", "hps_panel.cu", "hps_tc.cu", "hps_digit.cu", "hps_learned.cu", "hps_noalloc.cu", "hps_iface.cu", "hps_leaf2d.cu", "hps_cross.cu", "hps_iti.cu", "hps_assemble.cpp",
+SOURCES = ["hps_abi.cu", "hps_lu.cu", "hps_panel.cu", "hps_sweep.cu", "hps_tc.cu", "hps_digit.cu", "hps_learned.cu", "hps_noalloc.cu", "hps_iface.cu", "hps_leaf2d.cu", "hps_cross.cu", "hps_iti.cu", "hps_assemble.cpp",
            "hps_iface_plan.cpp", "hps_mixed.cpp", "hps_iti_host.cpp"]
 
 

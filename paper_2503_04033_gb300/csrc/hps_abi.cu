@@ -580,7 +580,8 @@ hps_status refine_chunk(hps_ctx* ctx, const Geometry& g, const CallSpec& cs, con
         } else
             launch_residual(g, cs.kappa, cs.kappa_dev, nbox, b, p3, cs.rhs_kind, cs.r, cs.rhs, cs.s_rhs, X, ldx, sX,
                             w.M + g.n, P.ldm, w.sM, w.skip, st, w.kb, cs.beta);
-        if (P.tc) {
+        if (narrow_solve(P, w, nbox, g.n, cs.r, w.skip, st)) {
+        } else if (P.tc) {
             if (!tc_lu_forward(P, w, nbox, g.n, cs.r, w.skip, st)) return HPS_ECUDA;
             if (!tc_lu_backward(P, w, nbox, g.n, cs.r, w.skip, st)) return HPS_ECUDA;
         } else {
@@ -944,8 +945,10 @@ hps_status factors_solve(hps_leaf_factors* F, int rhs_kind, int nrhs, const doub
     } else {
         if (F->P.tc) {
             tc_reset_abort(st);
-            if (!tc_lu_forward(F->P, w, nbox, n, nrhs, nullptr, st)) return HPS_ECUDA;
-            if (!tc_lu_backward(F->P, w, nbox, n, nrhs, nullptr, st)) return HPS_ECUDA;
+            if (!narrow_solve(F->P, w, nbox, n, nrhs, nullptr, st)) {
+                if (!tc_lu_forward(F->P, w, nbox, n, nrhs, nullptr, st)) return HPS_ECUDA;
+                if (!tc_lu_backward(F->P, w, nbox, n, nrhs, nullptr, st)) return HPS_ECUDA;
+            }
         } else {
             lu_forward<float>(F->P, w, nbox, n, nrhs, nullptr, st);
             lu_backward<float>(F->P, w, nbox, n, nrhs, nullptr, st);

@@ -5,6 +5,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <algorithm>
+#include <utility>
 #include <vector>
 
 #include "../../include/hps.h"
@@ -422,6 +423,11 @@ void tc_test_stall_next(int on);
 bool tc_test_stall_armed();
 bool tc_abort_raised();
 bool tc_lu_factor(const Plan& P, Work<float>& w, int nbox, int* status, cudaStream_t st);
+// Units of the tensor-core LU: (first step, steps).
+std::vector<std::pair<int, int>> lu_units(const Plan& P);
+// Forward and backward solve of up to eight columns [c0, c0 + nc) with the
+// FP32 joined operators (hps_sweep.cu); false when it does not apply.
+bool narrow_solve(const Plan& P, Work<float>& w, int nbox, int c0, int nc, const int* skip, cudaStream_t st);
 bool tc_lu_forward(const Plan& P, Work<float>& w, int nbox, int c0, int nc, const int* skip, cudaStream_t st);
 bool tc_lu_backward(const Plan& P, Work<float>& w, int nbox, int c0, int nc, const int* skip, cudaStream_t st);
 
