@@ -22,12 +22,14 @@
 // they displaced to the places that they left; perm[r] is the old row at
 // position r.
 //
-// What bounds it: with many boxes the multiply-adds of the elimination
-// (R nb^2 / 2 per box: the FP32 pipes at 128 a clock, the FP64 pipes at 2);
-// with few, the chain of nb pivots, about 500 clocks each with one CTA and
-// 1100 with a cluster, and the elimination divided by C.  Keeping rows in
-// registers leaves one shared-memory read of the pivot row per RPT rows where
-// a panel in shared memory took two reads and a write per multiply-add.
+// What bounds it: the chain of nb pivots with one box per CTA and SM (a barrier,
+// the comparison of eight offers and the first of the next column's entries per
+// pivot; a cluster adds its barrier, 390 clocks, and the exchange), and with many
+// boxes the issue of the elimination, R nb^2 / 2 multiply-adds.  Keeping rows in
+// registers leaves one shared-memory read of the pivot row per RPT rows where a
+// panel in shared memory took two reads and a write per multiply-add.  Against
+// that form: 128 columns of 1000 rows 475 -> 217 us (one box) and 1.94 -> 0.92 ms
+// (512 boxes); 64 FP64 columns of 216 rows 660 -> 160 us.
 #include <algorithm>
 #include <climits>
 #include <type_traits>
@@ -847,7 +849,8 @@ using PanelKernel = void (*)(const PanelArgs<T>);
 
 struct PanelShape {
     int rpt, ib;
-    int occ;   // CTAs per SM
+    int occ;        // CTAs per SM
+    double group;   // clocks of a pivot per group of 32 rows of an SM's CTAs
 };
 
 template <typename T>
@@ -875,8 +878,8 @@ PanelKernel<double> panel_kernel<double>(int i)
 template <typename T>
 PanelShape panel_shape(int i)
 {
-    static const PanelShape f[4] = {{1, 16, 2}, {2, 16, 2}, {4, 16, 2}, {8, 16, 1}};
-    static const PanelShape d[4] = {{1, 16, 2}, {2, 16, 1}, {4, 16, 1}, {8, 8, 1}};
+    static const PanelShape f[4] = {{1, 16, 2, 100}, {2, 16, 2, 100}, {4, 16, 2, 100}, {8, 16, 1, 125}};
+    static const PanelShape d[4] = {{1, 16, 2, 190}, {2, 16, 1, 240}, {4, 16, 1, 330}, {8, 8, 1, 380}};
     return sizeof(T) == 4 ? f[i] : d[i];
 }
 template <typename T>
@@ -902,10 +905,15 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
         return true;
     }();
     (void)once;
-    // Rows per thread and cluster size: the fewest waves of (chain of nb pivots
-    // + the elimination's issue).  Clocks of one pivot: about 500 alone and 1100
-    // in a cluster, and per group of 32 rows 25 (FP32) or 640 (FP64: 40
-    // multiply-adds of 64 clocks over four schedulers), shared by an SM's CTAs.
+    // Rows per thread and cluster size: the fewest waves of (chain of a pivot +
+    // the elimination's issue), in clocks fitted to timings of every shape at 1
+    // to 512 boxes and 64 to 5832 rows: the chain takes about 1500 alone and 2900
+    // in a cluster for FP32, 4300 and 6000 for FP64 (barriers, the offer, the
+    // left products' latency, spread over the pivots), and a group of 32 rows what
+    // panel_shape lists.  FP32, 128 columns: one box of 1000 rows 217 to 254 us
+    // by shape, 512 boxes of 2744 rows 3.6 ms with four CTAs of four rows a thread
+    // against 3.9 with two of eight; FP64, 64 columns: 8 boxes of 216 rows 160 us
+    // with one CTA a box against 204 with eight.
     const int R0 = n - k;
     int bi = 3, bc = kMaxCluster;
     double best = -1.0;
@@ -920,7 +928,8 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
             const double waves = (double)((ctas + slots - 1) / slots);
             const double share = (double)std::min<long long>(sh.occ, (ctas + 151) / 152);
             const double groups = (double)((R0 + 32 * c - 1) / (32 * c));
-            const double cost = waves * ((c == 1 ? 500.0 : 1100.0) + share * groups * (sizeof(T) == 4 ? 25.0 : 640.0));
+            const double chain = sizeof(T) == 4 ? (c == 1 ? 1500.0 : 2900.0) : (c == 1 ? 4300.0 : 6000.0);
+            const double cost = waves * (chain + share * groups * sh.group) + 0.2 * c;
             if (best < 0 || cost < best) { best = cost; bi = i; bc = c; }
         }
     }
