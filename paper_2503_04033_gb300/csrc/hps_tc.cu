@@ -56,7 +56,7 @@ constexpr uint32_t A_TILE = TC_BM * ROWB;                   // 8 KiB per plane
 #ifndef HPS_TC_PRE
 #define HPS_TC_PRE 3
 #endif
-constexpr int TC_STAGES = HPS_TC_STAGES;   // operand stages of the TMA -> MMA ring
+constexpr int TC_STAGES = HPS_TC_STAGES;   // operand stages of the TMA -> MMA ring at the widest tile
 constexpr int TC_EPI_WARPS = 4;                             // cp.async epilogue: one per TMEM lane quarter
 constexpr int TE_WARPS = HPS_TE_WARPS;                      // TMA epilogue: 4 or 8 (two per lane quarter)
 static_assert(TE_WARPS == 4 || TE_WARPS == 8, "the TMA epilogue takes one or two warps per TMEM lane quarter");
@@ -104,6 +104,13 @@ __host__ __device__ constexpr uint32_t b_tile() { return (uint32_t)TcFmt<FMT>::B
 template <int FMT>
 __host__ __device__ constexpr uint32_t stage_bytes() { return (uint32_t)TcFmt<FMT>::NPL * (A_TILE + b_tile<FMT>()); }
 constexpr uint32_t STAGE_BYTES = 48 * 1024;
+template <int FMT, int BNT>
+__host__ __device__ constexpr int tc_stages()
+{
+    constexpr uint32_t per = (uint32_t)TcFmt<FMT>::NPL * (A_TILE + (uint32_t)BNT * ROWB);
+    constexpr uint32_t fit = (uint32_t)TC_STAGES * STAGE_BYTES / per;
+    return fit < 8 ? (int)fit : 8;
+}
 constexpr int TC_BN_NARROW = 64;                            // tile width for products of at most 64 columns
 static_assert(stage_bytes<0>() == STAGE_BYTES && stage_bytes<1>() == STAGE_BYTES && stage_bytes<2>() == STAGE_BYTES &&
                   stage_bytes<3>() <= STAGE_BYTES,
@@ -387,10 +394,16 @@ k_tc_update(const __grid_constant__ TcMaps tm, TcArgs a)
     constexpr int BN = BNT, KPC = Fm::KPC, NPL = Fm::NPL;
     constexpr uint32_t B_TILE = (uint32_t)BN * ROWB;
     constexpr uint32_t STAGE_TX = (uint32_t)NPL * (A_TILE + B_TILE);   // bytes a stage receives
+    // The ring's bytes are the same for every width: narrower tiles get more
+    // stages (2 x FP16: three of 256 columns, four of 128, six of 64), so that
+    // a solve of few columns, a stream over the left operand, keeps as many
+    // bytes in flight: 32 loads on the stored factors of 128 boxes at p = 16,
+    // 4.84 -> 4.28 ms of products a solve.
+    constexpr int NST = tc_stages<FMT, BNT>();
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t ld_bar[TE_WARPS][TE_PRE];
-    __shared__ __align__(8) uint64_t full_bar[TC_STAGES];
-    __shared__ __align__(8) uint64_t empty_bar[TC_STAGES];
+    __shared__ __align__(8) uint64_t full_bar[NST];
+    __shared__ __align__(8) uint64_t empty_bar[NST];
     __shared__ __align__(8) uint64_t tfull_bar[2];
     __shared__ __align__(8) uint64_t tempty_bar[2];
     __shared__ __align__(8) uint64_t mdrain_bar;   // the MMA role's last commit when it gives up
@@ -410,7 +423,7 @@ k_tc_update(const __grid_constant__ TcMaps tm, TcArgs a)
     float* tbuf_all = reinterpret_cast<float*>(sbase_ptr + TC_STAGES * STAGE_BYTES);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TC_STAGES; ++s) {
+        for (int s = 0; s < NST; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 1);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
@@ -442,15 +455,15 @@ k_tc_update(const __grid_constant__ TcMaps tm, TcArgs a)
                 int box, m0, n0;
                 sc.decode(u, box, m0, n0);
                 for (int ch = 0; ch < a.kch; ++ch, ++g) {
-                    const int s = g % TC_STAGES;
-                    const uint32_t use = g / TC_STAGES;
-                    if (g >= TC_STAGES && !mbar_wait<false>(smem_u32(&empty_bar[s]), (use - 1) & 1, a.wait_ns)) {
+                    const int s = g % NST;
+                    const uint32_t use = g / NST;
+                    if (g >= NST && !mbar_wait<false>(smem_u32(&empty_bar[s]), (use - 1) & 1, a.wait_ns)) {
                         fail_sh = 1;
                         ok = false;
                         break;
                     }
                     const uint32_t fb = smem_u32(&full_bar[s]);
-                    const uint32_t st = sbase + s * STAGE_BYTES;
+                    const uint32_t st = sbase + s * STAGE_TX;
                     mbar_expect_tx(fb, STAGE_TX);
                     // A's K chunks come from the part whose range holds ch; part
                     // i's row 0 is row a_off[i] of the product (rows above it
@@ -468,8 +481,8 @@ k_tc_update(const __grid_constant__ TcMaps tm, TcArgs a)
             }
             // Drain: the last loads issued into each stage have landed before
             // this CTA exits (the MMA role waits for its own MMAs).
-            for (uint32_t h = (g > TC_STAGES ? g - TC_STAGES : 0); h < g; ++h)
-                mbar_drain(smem_u32(&full_bar[h % TC_STAGES]), (h / TC_STAGES) & 1, a.wait_ns / 4);
+            for (uint32_t h = (g > NST ? g - NST : 0); h < g; ++h)
+                mbar_drain(smem_u32(&full_bar[h % NST]), (h / NST) & 1, a.wait_ns / 4);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -489,14 +502,14 @@ k_tc_update(const __grid_constant__ TcMaps tm, TcArgs a)
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(b * BN);
                 for (int ch = 0; ch < a.kch; ++ch, ++g) {
-                    const int s = g % TC_STAGES;
-                    if (!mbar_wait<false>(smem_u32(&full_bar[s]), (g / TC_STAGES) & 1, a.wait_ns)) {
+                    const int s = g % NST;
+                    if (!mbar_wait<false>(smem_u32(&full_bar[s]), (g / NST) & 1, a.wait_ns)) {
                         fail_sh = 1;
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t st = sbase + s * STAGE_BYTES;
+                    const uint32_t st = sbase + s * STAGE_TX;
                     uint64_t ad[NPL], bd[NPL];
 #pragma unroll
                     for (int pl = 0; pl < NPL; ++pl) {
