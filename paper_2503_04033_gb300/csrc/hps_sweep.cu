@@ -1,15 +1,15 @@
 // Triangular solves of a few right-hand sides with the joined LU operators.
 //
-// A refinement or a time step solves for one to eight columns per box: a
+// A refinement or a time step solves for one to four columns per box: a
 // product of a unit then reads its operator once (4 bytes an entry, 2 MB a box
-// and direction at n = 1000) for at most eight multiply-adds, so the sweep is a
+// and direction at n = 1000) for at most four multiply-adds, so the sweep is a
 // stream over the FP32 operators F and B, bound by HBM.  The tensor-core form
 // pads the columns to 64, gathers them into packed operands first and took 43 us
 // + 8 us (gather) for the first unit of 64 boxes at n = 1000, one column, where
 // the stream needs 20 at 6.8 TB/s.
 //
 // Each launch applies one unit: a CTA stages the unit's block of pivot rows (at
-// most 1024 x 8 values) in shared memory, and every warp takes four rows of the
+// most 1024 x 4 values) in shared memory, and every warp takes four rows of the
 // operator at a time, 16 bytes a lane, so that a warp has up to 16 loads in
 // flight.  Source and result are different buffers (the columns of M at the
 // ends, two compact [row][column] buffers between), so no rows are saved and no
@@ -140,8 +140,7 @@ void launch_sweep(const SweepArgs& a, int nbox, cudaStream_t st)
     prof_begin(cls, st);
     if (a.N == 1) go(k_sweep<1>, 1);
     else if (a.N == 2) go(k_sweep<2>, 2);
-    else if (a.N <= 4) go(k_sweep<4>, 4);
-    else go(k_sweep<8>, 8);
+    else go(k_sweep<4>, 4);
     double el = 0.0;
     for (int p = 0; p < a.nparts; ++p) el += (double)a.rows[p] * a.K[p];
     prof_end(cls, st, 2.0 * nbox * el * a.N, (double)nbox * el * 4.0);
@@ -151,7 +150,12 @@ void launch_sweep(const SweepArgs& a, int nbox, cudaStream_t st)
 
 bool narrow_solve(const Plan& P, Work<float>& w, int nbox, int c0, int nc, const int* skip, cudaStream_t st)
 {
-    if (!P.tc || nc > 8 || P.unit_max > SW_PARTS) return false;
+    // Four columns is the line: solves with stored factors take, streamed against
+    // tensor-core, 536 : 1044 us for one column, 657 : 1087 for four and 1276 :
+    // 1118 for eight (64 boxes at p = 12), 2973 : 5800, 4352 : 5937 and 9677 : 6209
+    // (128 boxes at p = 16): eight columns' accumulators and their reads of the
+    // staged block outgrow the stream.
+    if (!P.tc || nc > 4 || P.unit_max > SW_PARTS) return false;
     const auto units = lu_units(P);
     const int U = (int)units.size(), total = 2 * U;
     if ((size_t)P.n * nc * sizeof(float) > P.bW) return false;   // the compact buffers are W and W2

@@ -1,6 +1,6 @@
 """Few right-hand sides through the streamed sweeps: every column count they
-take (1 .. 8, with the padded ones 3, 5 and 7) and the first that they leave to
-the tensor-core products (9), at orders whose LU has one ragged unit (p = 5, 8),
+take (1 .. 4, with the padded 3) and some that they leave to the tensor-core
+products (5 .. 9), at orders whose LU has one ragged unit (p = 5, 8),
 a ragged last step (p = 9: 343 = 2 x 128 + 87) and several units (p = 12, 13).
 Reference: the FP64 path's solves of the same boxes; both forms refine to
 1e-11 of the solution, so they agree to 1e-10."""
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("p", [5, 8, 9, 12, 13])
-@pytest.mark.parametrize("nrhs", [1, 2, 3, 5, 7, 8, 9])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 4, 5, 7, 8, 9])
 def test_few_columns_match_fp64(p, nrhs):
     import torch
     import paper_2503_04033_gb300 as H
