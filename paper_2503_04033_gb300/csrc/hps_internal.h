@@ -150,6 +150,7 @@ inline Plan make_plan(int n, int r, hps_precision prec, int nb_opt, bool use_tc,
     int NB = nb_opt > 0 ? nb_opt : (fp64 ? 64 : 128);
     if (fp64 && NB > 64) NB = 64;
     if (NB > kMaxNB) NB = kMaxNB;
+    NB = (int)align_up((size_t)NB, 16);   // the panel's 16-byte accesses; options and tuned plans are 32, 64 or 128
     P.NB = NB;
     P.ldm = (long long)align_up((size_t)(n + r), 8);
     for (int k = 0; k < n; k += NB) {
@@ -425,7 +426,7 @@ bool tc_abort_raised();
 bool tc_lu_factor(const Plan& P, Work<float>& w, int nbox, int* status, cudaStream_t st);
 // Units of the tensor-core LU: (first step, steps).
 std::vector<std::pair<int, int>> lu_units(const Plan& P);
-// Forward and backward solve of up to eight columns [c0, c0 + nc) with the
+// Forward and backward solve of up to four columns [c0, c0 + nc) with the
 // FP32 joined operators (hps_sweep.cu); false when it does not apply.
 bool narrow_solve(const Plan& P, Work<float>& w, int nbox, int c0, int nc, const int* skip, cudaStream_t st);
 bool tc_lu_forward(const Plan& P, Work<float>& w, int nbox, int c0, int nc, const int* skip, cudaStream_t st);
