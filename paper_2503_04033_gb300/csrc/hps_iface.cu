@@ -596,14 +596,21 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     // 16-byte aligned (e a multiple of 4: every even q) and the product pays for
     // its two packs (1e8 multiply-adds take the CUDA cores 12 us), on the CUDA
     // cores elsewhere.  8 x 8 x 8 boxes at p = 12: 145 ms on the CUDA cores, 17 ms with
-    // the operand packs.
-    const bool tc_merge = sizeof(MT) == 4 && e > 0 && e % 4 == 0 && (double)L.nn * e * e * s >= 1e8;
+    // the operand packs.  Without room for the packs the CUDA cores take it too.
+    bool tc_merge = sizeof(MT) == 4 && e > 0 && e % 4 == 0 && (double)L.nn * e * e * s >= 1e8;
     const size_t lu_bytes = PL.per_box * (size_t)L.nn;
     const size_t merge_bytes = tc_merge ? hps::tc_gemm_f32_scratch(e, e, s) * (size_t)L.nn : 0;
-    const size_t need = hps::align_up(lu_bytes, 1024) + merge_bytes;
+    size_t need = hps::align_up(lu_bytes, 1024) + merge_bytes;
     if (need > *ws_bytes) {
         if (*ws) { cudaStreamSynchronize(st); cudaFree(*ws); *ws = nullptr; *ws_bytes = 0; }
-        if (cudaMalloc(ws, need) != cudaSuccess) { cudaGetLastError(); return HPS_ENOMEM; }
+        if (cudaMalloc(ws, need) != cudaSuccess) {
+            cudaGetLastError();
+            *ws = nullptr;
+            if (!tc_merge) return HPS_ENOMEM;
+            tc_merge = false;
+            need = lu_bytes;
+            if (cudaMalloc(ws, need) != cudaSuccess) { cudaGetLastError(); *ws = nullptr; return HPS_ENOMEM; }
+        }
         *ws_bytes = need;
     }
     if ((size_t)L.nn > *status_cap) {
