@@ -22,7 +22,8 @@
 // So the only roundings are those three; a plain FP64 sum rounds K times.
 // Against a higher-precision solve, the LU built on these products is as close
 // as or closer than the one on FP64 multiply-adds (tests/test_gpu_digit.py).
-// A row or column that holds an infinity or a NaN gives NaN throughout.
+// Results outside the normal range, and all of a row or column that holds an
+// infinity or a NaN, are summed as they stand on the FP64 pipe instead.
 //
 // Layout.  One CTA of 512 threads per SM takes a 128-row strip of A (split
 // once, 128 KiB of digits in shared memory) across a range of column tiles of
@@ -41,7 +42,7 @@
 // or by a warp of their own were each slower (2.0, 2.4 and 2.6 ms against 1.74):
 // they cost registers or coalesced reads of B, and the MMAs' latency shows.
 // Whole calls: 512 boxes at p = 12 (DtN, particular and reconstruction) 1001 ->
-// 102 ms, cross-term leaves 225 -> 34 ms.
+// 101 ms, cross-term leaves 225 -> 39 ms.
 #include <algorithm>
 
 #include "hps_digits.cuh"
@@ -115,10 +116,29 @@ __device__ __forceinline__ void split_to(const double (&x)[4], int E, unsigned c
     for (int s = 0; s < DG_S; ++s) *reinterpret_cast<uint2*>(base + s * plane) = make_uint2(d[s][0], d[s][1]);
 }
 
+// The rare results (round_fixed asked for another look): this lane's row times
+// column `col` of the CTA's range, as they stand, on the FP64 pipe.  Everything
+// is taken from the arguments again, so that the main path keeps nothing for it.
+template <bool BT>
+__device__ __noinline__ double plain_sum(const DgArgs& a, int col)
+{
+    const GemmArgs<double>& g = a.g;
+    const int warp = threadIdx.x >> 5;
+    const int r = blockIdx.y * DG_BM + (warp & 3) * 32 + (threadIdx.x & 31);
+    const int c = blockIdx.x * a.per * DG_BN + (warp >> 2) * 8 + col;
+    if (r >= g.M || c >= g.N) return 0.0;
+    const double* x = g.A + blockIdx.z * g.sA + r * g.lda;
+    const double* y = g.B + blockIdx.z * g.sB + (BT ? c * g.ldb : c);
+    const long long step = BT ? 1 : g.ldb;
+    double s = 0.0;
+    for (int k = 0; k < g.K; ++k) s = fma(x[k], y[k * step], s);
+    return s;
+}
+
 // BT: B is given transposed, [n][k] with k contiguous.
 template <bool BT>
 __global__ void __launch_bounds__(DG_THREADS, 1)
-k_digit_gemm(const DgArgs a)
+k_digit_gemm(const __grid_constant__ DgArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t tfull[2];   // a tile's accumulators are complete
@@ -302,10 +322,9 @@ k_digit_gemm(const DgArgs a)
             }
             if (odd) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    double& r = st[lane * 8 + ((h + c) ^ ((lane >> 1) & 7))];
-                    r = finish_odd(r, E[c], eb[c]);
-                }
+                for (int c = 0; c < 4; ++c)
+                    if ((unsigned)eb[c] > 2045u)
+                        st[lane * 8 + ((h + c) ^ ((lane >> 1) & 7))] = plain_sum<BT>(a, j * DG_BN + h + c);
             }
         }
         __syncwarp();
