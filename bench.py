@@ -1273,8 +1273,8 @@ def run_leaf2d(args):
             "tflops": tflops,
             "roofline": {"bound": "alu", "achieved": tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": tflops / FP64_PEAK_TFLOPS, "traffic": None,
-                         "peak_source": "FP64 issue rate 152 SMs x 2.07 GHz x 2 FMA/clk (the whole call, its LU "
-                                        "on the CUDA-core FP64 path)"},
+                         "peak_source": "FP64 issue rate 152 SMs x 2.07 GHz x 2 FMA/clk (the whole call; its LU products "
+                                        "run from exact digits on the tensor cores, so frac can pass 1)"},
             "rel_err_vs_oracle_max": worst, "box_failures": fails, "clocks": clocks.summary(),
             "cpu_baseline": {"value": len(sel) / cpu_s, "unit": "boxes/s", "cores": oracle.max_threads(),
                              "kind": "oracle", "sample": f"{len(sel)} boxes spread over the grid, 2-D FP64 oracle "
@@ -1293,8 +1293,8 @@ def _fp64_leaf_line(metric, value, ms, args, workload, flops_per_box, worst, fai
             "tflops": tflops,
             "roofline": {"bound": "alu", "achieved": tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                          "frac": tflops / FP64_PEAK_TFLOPS, "traffic": None,
-                         "peak_source": "FP64 issue rate 152 SMs x 2.07 GHz x 2 FMA/clk (the whole call, its LU "
-                                        "on the CUDA-core FP64 path)"},
+                         "peak_source": "FP64 issue rate 152 SMs x 2.07 GHz x 2 FMA/clk (the whole call; its LU products "
+                                        "run from exact digits on the tensor cores, so frac can pass 1)"},
             "rel_err_vs_oracle_max": worst, "box_failures": fails, "clocks": clocks.summary(),
             "cpu_baseline": {"value": cpu_rate, "unit": "boxes/s", "cores": oracle.max_threads(), "kind": "oracle",
                              "sample": f"{cpu_n} boxes spread over the batch, FP64 oracle, one box at a time"}}

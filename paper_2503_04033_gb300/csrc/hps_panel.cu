@@ -933,7 +933,9 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
             if (best < 0 || cost < best) { best = cost; bi = i; bc = c; }
         }
     }
-    // the multipliers' scratch is the step's F block, which the inverse and the
+    // Rows are read and written 16 bytes at a time: M is 256-byte aligned, ldm a
+    // multiple of 8 and k one of 16 (make_plan rounds every stride up, steps are
+    // NB wide).  The multipliers' scratch is the step's F block, which the inverse and the
     // product after this overwrite
     PanelArgs<T> a{M, ldm, sM, n, k, nb, Ftop, sF, perm, sP, status, skip};
     prof_begin(KC_PANEL, st);
