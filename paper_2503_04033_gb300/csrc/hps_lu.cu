@@ -1267,28 +1267,14 @@ void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c
     prof_end(KC_GATHER, st, 0.0, (double)nbox * nb * (double)ncols * sizeof(T) * (W ? 3 : 2));
 }
 
-// FP64 products of at least this many multiply-adds per box run from exact
-// digits on the tensor cores.  The rule depends on one box's sizes only, so a
-// batch and its chunks take the same arithmetic.  p = 5 (27 x 54 x 27): 341 us
-// a call on the FP64 pipes, 283 us from digits, for 1 to 64 boxes alike.
-#ifndef HPS_DIGIT_MIN
-#define HPS_DIGIT_MIN 4096.0
-#endif
-constexpr double kDigitMin = HPS_DIGIT_MIN;
-
+// FP64 products run from exact digits on the tensor cores at every size, the
+// smallest included: 4096 boxes at p = 3 (products of 1 x 6 x 1) take 1000 us a
+// call against 1390 on the FP64 pipes, p = 4 (8 x 24 x 8) 1267 : 1677, p = 5
+// 2610 : 3692, one box at p = 5 117 : 173, with errors of T no larger.
 template <>
 void launch_gemm<double>(const GemmArgs<double>& a, int nbox, cudaStream_t st)
 {
-    constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
-    dim3 grd((unsigned)((a.N + BN - 1) / BN), (unsigned)((a.M + BM - 1) / BM), (unsigned)nbox);
-    if (a.M <= 0 || a.N <= 0) return;
-    if ((double)a.M * a.N * a.K >= kDigitMin) {
-        launch_digit_gemm(a, false, nbox, st);
-        return;
-    }
-    prof_begin(KC_UPDATE_CUDACORE, st);
-    k_gemm<double, BM, BN, BK, TM, TN><<<grd, (BM / TM) * (BN / TN), 0, st>>>(a);
-    prof_end(KC_UPDATE_CUDACORE, st, 2.0 * nbox * a.M * (double)a.N * a.K, (double)nbox * ((double)a.M * a.K + (double)a.K * a.N + 2.0 * a.M * a.N) * 8);
+    launch_digit_gemm(a, false, nbox, st);
 }
 
 template <>
