@@ -564,7 +564,7 @@ k_tc_update(const __grid_constant__ TcMaps tm, TcArgs a)
         // replaces the staged row by src - acc in place (128B swizzle: 16-byte
         // unit u of row r sits at u ^ (r % 8), so a quarter-warp touches 8
         // distinct bank groups) and lane 0 stores the chunk back by TMA, which
-        // clips at O's edge.  Rows whose source is zero (SET, the pivot block
+        // clips at the 16-byte unit that holds O's edge.  Rows whose source is zero (SET, the pivot block
         // in FWD, below the split in BWD) or a saved row W (FWD rows whose
         // pivot source lies above the split) ignore the staged row.
         const int qd = warp & 3, ew = warp - 2;
@@ -1359,6 +1359,10 @@ bool launch_tc_update_w(const TcLeft& L, const void* Gp, long long g_plane, long
     const auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     a.vec = al16(a.O) && (a.ldo % 4 == 0) && (a.sO % 4 == 0) && (a.N % 4 == 0) &&
             (!a.W || (al16(a.W) && a.ldw % 4 == 0 && a.sW % 4 == 0));
+    // A TMA store writes whole 16-byte units: where N is no multiple of 4 it also
+    // zeroes the entries between O's last column and the next 16-byte boundary
+    // (measured: a map of 41 columns writes 41 .. 43 as well).  Padding may lie
+    // there, live columns may not: the caller then passes allow_tma false.
     a.tma_epi = 0;
     if (al16(a.O) && a.ldo % 4 == 0 && a.sO % 4 == 0 && allow_tma) {
         auto fn = encode_fn();
@@ -1685,10 +1689,10 @@ bool tc_lu_factor(const Plan& P, Work<float>& w, int nbox, int* status, cudaStre
 {
     const int n = P.n, NB = P.NB, KG = P.KG;
     const long long ldm = P.ldm, gplane = ldm * KG;
-    auto up = [&](const TcLeft& L, TcArgs a) {
+    auto up = [&](const TcLeft& L, TcArgs a, bool allow_tma = true) {
         a.invt = w.it1;
         a.sInvt = w.sIT;
-        return launch_tc_update(P.fmt, L, w.Gp, gplane, w.sGp, KG, NB, a, nbox, st, P.tma_epi, P.bn_max);
+        return launch_tc_update(P.fmt, L, w.Gp, gplane, w.sGp, KG, NB, a, nbox, st, P.tma_epi && allow_tma, P.bn_max);
     };
     // Panel of step s, its operators F_s and B_s (FP32 and split copies; B_s's
     // split only when pack_b: a B part that a join rewrites before any
@@ -1734,7 +1738,8 @@ bool tc_lu_factor(const Plan& P, Work<float>& w, int nbox, int* status, cudaStre
         launch_gather_pack(P, w, k, wp, c0, nc, Ps, true, nullptr, nbox, st, rcf(P, w, s));
         TcArgs a = targs(w.M + (long long)k * ldm + c0, ldm, w.sM, n - k, nc, GM_FWD, wp);
         a.perm = Ps; a.sP = w.sP; a.W = w.W; a.ldw = ldm; a.sW = w.sG; a.status = status;
-        return up(left_fwd(P, w, s, len), a);
+        // columns that end inside a 16-byte unit of M with right-hand sides in its rest: no TMA stores
+        return up(left_fwd(P, w, s, len), a, nc % 4 == 0 || c0 + nc == n + P.r);
     };
     // Join the units A = (s, h) and B = (s + h, h) into (s, 2 h).
     auto join = [&](int s, int h) -> bool {
