@@ -591,26 +591,10 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     // FP64 refinement recovers the digits
     const bool tc = sizeof(MT) == 4 && s >= 256;
     hps::Plan PL = hps::make_plan(s, e + s, tc ? HPS_BF16_IR : prec, 0, tc, false);
-    // The merged maps' products E S in FP32: with 3 x BF16 operands (FP32's 24
-    // bits, FP32 accumulation) on the tensor cores where the map's rows are
-    // 16-byte aligned (e a multiple of 4: every even q) and the product pays for
-    // its two packs (1e8 multiply-adds take the CUDA cores 12 us), on the CUDA
-    // cores elsewhere.  8 x 8 x 8 boxes at p = 12: 145 ms on the CUDA cores, 17 ms with
-    // the operand packs.  Without room for the packs the CUDA cores take it too.
-    bool tc_merge = sizeof(MT) == 4 && e > 0 && e % 4 == 0 && (double)L.nn * e * e * s >= 1e8;
-    const size_t lu_bytes = PL.per_box * (size_t)L.nn;
-    const size_t merge_bytes = tc_merge ? hps::tc_gemm_f32_scratch(e, e, s) * (size_t)L.nn : 0;
-    size_t need = hps::align_up(lu_bytes, 1024) + merge_bytes;
+    const size_t need = PL.per_box * (size_t)L.nn;
     if (need > *ws_bytes) {
         if (*ws) { cudaStreamSynchronize(st); cudaFree(*ws); *ws = nullptr; *ws_bytes = 0; }
-        if (cudaMalloc(ws, need) != cudaSuccess) {
-            cudaGetLastError();
-            *ws = nullptr;
-            if (!tc_merge) return HPS_ENOMEM;
-            tc_merge = false;
-            need = lu_bytes;
-            if (cudaMalloc(ws, need) != cudaSuccess) { cudaGetLastError(); *ws = nullptr; return HPS_ENOMEM; }
-        }
+        if (cudaMalloc(ws, need) != cudaSuccess) { cudaGetLastError(); *ws = nullptr; return HPS_ENOMEM; }
         *ws_bytes = need;
     }
     if ((size_t)L.nn > *status_cap) {
@@ -642,16 +626,10 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     k_if_extract<MT><<<dim3((unsigned)s, (unsigned)L.nn), 256, 0, st>>>(w.M, PL.ldm, w.sM, s, e,
                                                                          static_cast<MT*>(L.S),
                                                                          static_cast<MT*>(L.Winv));
-    if constexpr (sizeof(MT) == 4) {
-        if (tc_merge) {   // Tn -= E X with X = -S, the solved columns of M
-            if (!tc_done) hps::tc_reset_abort(st);
-            if (!hps::tc_gemm_f32(e, e, s, static_cast<const float*>(L.E), s, (long long)e * s, w.M + s, PL.ldm, w.sM,
-                                  static_cast<float*>(L.Tn), e, (long long)e * e, *d_status, L.nn,
-                                  static_cast<char*>(*ws) + hps::align_up(lu_bytes, 1024), st))
-                return HPS_ECUDA;
-        }
-    }
-    if (e > 0 && !tc_merge)
+    // FP32 multiply-adds also in FP32: summed by the tensor cores from 3 x BF16
+    // operands (17 ms instead of 145 for 8 x 8 x 8 boxes at p = 12) the maps were
+    // 3 to 20 times further from 64 bits, the accumulators being cut, not rounded
+    if (e > 0)
         if_merge_product<MT>(L.nn, e, s, static_cast<const MT*>(L.E), static_cast<const MT*>(L.S),
                              static_cast<MT*>(L.Tn), st);
     if (cudaGetLastError() != cudaSuccess) return HPS_ECUDA;

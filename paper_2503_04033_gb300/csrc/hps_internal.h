@@ -409,12 +409,6 @@ void lu_backward(const Plan& P, Work<T>& w, int nbox, int c0, int nc, const int*
 // described to TMA.
 bool tc_gemm_bf16(int M, int N, int K, const void* A, long long lda, long long sA, const void* B, long long ldb,
                   long long sB, float* C, long long ldc, long long sC, bool accumulate, int batch, cudaStream_t st);
-// C -= A B per batch entry in FP32 with 3 x BF16 operands; scratch holds
-// tc_gemm_f32_scratch bytes per entry.
-size_t tc_gemm_f32_scratch(int M, int N, int K);
-bool tc_gemm_f32(int M, int N, int K, const float* A, long long lda, long long sA, const float* B, long long ldb,
-                 long long sB, float* C, long long ldc, long long sC, int* status, int batch, void* scratch,
-                 cudaStream_t st);
 void tc_reset_abort(cudaStream_t st);
 
 // Test hook: the next tensor-core launch of a call that writes box status

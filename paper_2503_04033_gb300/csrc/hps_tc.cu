@@ -1518,34 +1518,6 @@ bool tc_gemm_bf16(int M, int N, int K, const void* A, long long lda, long long s
     return launch_tc_update_f<3>(L, B, (long long)N * ldb, sB, K, K, a, batch, st, true, 256, nullptr, ldb);
 }
 
-size_t tc_gemm_f32_scratch(int M, int N, int K)
-{
-    return align_up((size_t)3 * 2 * align_up((size_t)K, 32) * M, 256) +
-           align_up((size_t)3 * 2 * align_up((size_t)K, 32) * N, 256);
-}
-
-// C -= A B per batch entry, FP32 row-major, on tcgen05 with 3 x BF16 operands
-// (format 1) and FP32 accumulation: A is split into the scratch's first part,
-// B transposed and split into its second.
-bool tc_gemm_f32(int M, int N, int K, const float* A, long long lda, long long sA, const float* B, long long ldb,
-                 long long sB, float* C, long long ldc, long long sC, int* status, int batch, void* scratch,
-                 cudaStream_t st)
-{
-    if (K <= 0) return false;
-    const int Kp = (int)align_up((size_t)K, 32);
-    const size_t per = tc_gemm_f32_scratch(M, N, K), perA = align_up((size_t)6 * Kp * M, 256);
-    unsigned short* Ap = static_cast<unsigned short*>(scratch);
-    unsigned short* Bp = Ap + (perA * (size_t)batch) / 2;
-    const long long sAp = (long long)(perA / 2), sBp = (long long)((per - perA) / 2);
-    launch_pack_split(1, A, lda, sA, M, Kp, K, Ap, sAp, batch, st);
-    gather_pack_raw(1, B, ldb, sB, 0, K, Kp, 0, N, nullptr, 0, nullptr, 0, 0, Bp, (long long)N * Kp, sBp, nullptr, batch,
-                    st);
-    TcArgs a = targs(C, ldc, sC, M, N, GM_ACC, 0);
-    a.status = status;
-    return launch_tc_update_f<1>(left1(Ap, M, sAp, K), Bp, (long long)N * Kp, sBp, Kp, Kp, a, batch, st, true, 256,
-                                 nullptr);
-}
-
 void tc_test_stall_next(int on) { g_test_stall_next = on ? 1 : 0; }
 bool tc_test_stall_armed() { return g_test_stall_next != 0; }
 
