@@ -72,7 +72,14 @@ typedef enum {
 } hps_status;
 
 /* Arithmetic of the LU and the triangular solves.  HPS_FP64 runs everything
- * in FP64 (the plain path).  HPS_FP32_IR factors A_ii in FP32 on the tensor
+ * in FP64 (the plain path).  Its products are summed exactly from 8-bit digits
+ * of the operands, fixed point under one power of two per row and column: off by
+ * about 2^-58 (2^-51 at worst) of the largest entry of the row times that of the
+ * column, where an FP64 sum is off by some 2^-53 of its terms.  A matrix whose
+ * rows' largest entries lie 2^9 or more apart (coefficients that jump by 1e7 and
+ * more inside a box), or a box whose axes' second differences do by 2^12 (sides
+ * 1 : 64), is factored and solved on plain FP64 sums instead, about nine times
+ * slower.  HPS_FP32_IR factors A_ii in FP32 on the tensor
  * cores (3-term TF32 split products with FP32 accumulation) and recovers FP64
  * accuracy by iterative refinement: residuals R = -A_ib - A_ii X computed
  * matrix-free in FP64, corrections solved with the FP32 factors, X updated in
@@ -287,7 +294,8 @@ hps_status hps_mlp_grad_target(hps_mlp* net, int B, const double* b_in, const fl
 /* One Adam update with the last gradients. */
 hps_status hps_mlp_adam_step(hps_mlp* net, float lr, float beta1, float beta2, float eps, void* stream);
 
-/* T[b] = T0 + scale U[b] V[b]^T (device, FP64; T0 [m][m] shared). */
+/* T[b] = T0 + scale U[b] V[b]^T (device, FP64; T0 [m][m] shared).  Every entry of
+ * U V^T is within the error bound of an FP64 sum, rank 2^-53 sum |u||v|. */
 hps_status hps_lowrank_dtn(int nbox, int m, int rank, const double* T0, double scale, const double* U,
                            const double* V, double* T, void* stream);
 

@@ -183,10 +183,11 @@ void cheb_diff(int p, double* D)
 // ------------------------------------------------------------ LU sequences
 
 template <typename T>
-GemmArgs<T> gargs()
+GemmArgs<T> gargs(const Work<T>& w)
 {
     GemmArgs<T> a{};
     a.alpha = T(-1);
+    a.wide = w.wide;
     return a;
 }
 
@@ -197,15 +198,16 @@ void lu_factor(const Plan& P, Work<T>& w, int nbox, int* status, cudaStream_t st
 {
     const int n = P.n, NB = P.NB;
     const long long ldm = P.ldm;
+    if constexpr (sizeof(T) == 8) launch_wide(w.M, ldm, w.sM, n, P.axis, P.dims, w.wide, nbox, st);
     for (int s = 0; s < P.nsteps; ++s) {
         const int k = P.k0[s], nb = P.nbs[s];
         T* Fs = w.F + P.fw_off[s];
         T* Bs = w.B + P.bw_off[s];
         int* Ps = w.perm + P.perm_off[s];
         launch_panel<T>(w.M, ldm, w.sM, n, k, nb, Ps, w.sP, Fs, NB, w.sF, Bs + (long long)k * NB, NB, w.sB,
-                        status, nullptr, nbox, st);
+                        status, nullptr, w.wide, nbox, st);
         if (n - k - nb > 0) {
-            GemmArgs<T> a = gargs<T>();
+            GemmArgs<T> a = gargs<T>(w);
             a.A = w.M + (long long)(k + nb) * ldm + k; a.lda = ldm; a.sA = w.sM;
             a.B = Fs; a.ldb = NB; a.sB = w.sF;
             a.O = Fs + (long long)nb * NB; a.ldo = NB; a.sO = w.sF;
@@ -213,7 +215,7 @@ void lu_factor(const Plan& P, Work<T>& w, int nbox, int* status, cudaStream_t st
             launch_gemm<T>(a, nbox, st);
         }
         if (k > 0) {
-            GemmArgs<T> a = gargs<T>();
+            GemmArgs<T> a = gargs<T>(w);
             a.A = w.M + k; a.lda = ldm; a.sA = w.sM;
             a.B = Bs + (long long)k * NB; a.ldb = NB; a.sB = w.sB;
             a.O = Bs; a.ldo = NB; a.sO = w.sB;
@@ -223,7 +225,7 @@ void lu_factor(const Plan& P, Work<T>& w, int nbox, int* status, cudaStream_t st
         const int c0 = k + nb, nc = n + P.r - c0;
         if (nc > 0) {
             launch_gather<T>(w.M, ldm, w.sM, k, nb, c0, nc, Ps, w.sP, w.W, w.G, ldm, w.sG, nullptr, nbox, st);
-            GemmArgs<T> a = gargs<T>();
+            GemmArgs<T> a = gargs<T>(w);
             a.A = Fs; a.lda = NB; a.sA = w.sF;
             a.B = w.G; a.ldb = ldm; a.sB = w.sG;
             a.O = w.M + (long long)k * ldm + c0; a.ldo = ldm; a.sO = w.sM;
@@ -245,7 +247,7 @@ void lu_forward(const Plan& P, Work<T>& w, int nbox, int c0, int nc, const int* 
         T* Fs = w.F + P.fw_off[s];
         int* Ps = w.perm + P.perm_off[s];
         launch_gather<T>(w.M, ldm, w.sM, k, nb, c0, nc, Ps, w.sP, w.W, w.G, ldm, w.sG, skip, nbox, st);
-        GemmArgs<T> a = gargs<T>();
+        GemmArgs<T> a = gargs<T>(w);
         a.A = Fs; a.lda = NB; a.sA = w.sF;
         a.B = w.G; a.ldb = ldm; a.sB = w.sG;
         a.O = w.M + (long long)k * ldm + c0; a.ldo = ldm; a.sO = w.sM;
@@ -265,7 +267,7 @@ void lu_backward(const Plan& P, Work<T>& w, int nbox, int c0, int nc, const int*
         const int k = P.k0[s], nb = P.nbs[s];
         T* Bs = w.B + P.bw_off[s];
         launch_gather<T>(w.M, ldm, w.sM, k, nb, c0, nc, nullptr, 0, nullptr, w.G, ldm, w.sG, skip, nbox, st);
-        GemmArgs<T> a = gargs<T>();
+        GemmArgs<T> a = gargs<T>(w);
         a.A = Bs; a.lda = NB; a.sA = w.sB;
         a.B = w.G; a.ldb = ldm; a.sB = w.sG;
         a.O = w.M + c0; a.ldo = ldm; a.sO = w.sM;
@@ -406,6 +408,8 @@ Plan job_plan(const hps_ctx* ctx, const Job& j, hps_precision prec)
 {
     Plan P = make_plan(j.g->n, job_cols(j), prec, j.nb ? j.nb : ctx->nb_opt, ctx->use_tc != 0, prec != HPS_FP64,
                        j.unit ? j.unit : ctx->lu_unit, ctx->fp16_ops != 0);
+    P.axis = j.g->q;
+    P.dims = 3;
     P.bn_max = j.bn ? j.bn : 256;
     P.tma_epi = ctx->tc_epi_cp == 0;
     if (ctx->tc_fuse >= 0) P.fuse_bwd = P.tc && ctx->tc_fuse != 0;

@@ -393,6 +393,8 @@ hps_status hps_leaf_cross_solve(int p, const double h[3], double kappa, int nbox
     small.insert(small.end(), tab.G.begin(), tab.G.end());
     small.insert(small.end(), tab.Q.begin(), tab.Q.end());
     hps::Plan PL = hps::make_plan(n, m + nrhs, HPS_FP64, 0, false, false);
+    PL.axis = p - 2;
+    PL.dims = 3;
     const size_t small_bytes = hps::align_up(sizeof(double) * small.size(), 256);
     const size_t te_bytes = hps::align_up(sizeof(double) * tab.TE.size(), 256);
     const size_t st_bytes = hps::align_up(sizeof(int) * (size_t)nbox, 256);

@@ -19,7 +19,9 @@
 //     were largest and of one sign) are joined in 64-bit integers with a unit
 //     of 2^-57, rounded once to FP64 and added to the source.
 //
-// So the only roundings are those three; a plain FP64 sum rounds K times.
+// So the only roundings are those three; a plain FP64 sum rounds K times, but
+// relative to its own terms, not to the scales: operands whose scales say little
+// about an entry are summed plainly on the FP64 pipe (CHECK below, launch_wide).
 // Against a higher-precision solve, the LU built on these products is as close
 // as or closer than the one on FP64 multiply-adds (tests/test_gpu_digit.py).
 // Results outside the normal range, and all of a row or column that holds an
@@ -66,6 +68,7 @@ constexpr uint64_t DG_WAIT_NS = 2000000000ull;
 struct DgArgs {
     GemmArgs<double> g;
     int tiles_n, per;   // column tiles, and how many of them a CTA takes
+    int reach;          // CHECK: an entry's large factors are those within 2^-reach of their scales
 };
 
 // Sum of acc_t 2^(45 - 8 t) (unit 2^-57 of the scales' product 2^(E - 1016 ..))
@@ -135,8 +138,110 @@ __device__ __noinline__ double plain_sum(const DgArgs& a, int col)
     return s;
 }
 
-// BT: B is given transposed, [n][k] with k contiguous.
+// The same for the entries of the warp's 32 x 8 block that are set in `fix` (a
+// bit per column), a row a lane.
 template <bool BT>
+__device__ __noinline__ void plain_block(const DgArgs& a, int col, double* st, uint32_t fix)
+{
+    const GemmArgs<double>& g = a.g;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c0 = blockIdx.x * a.per * DG_BN + (warp >> 2) * 8 + col;
+    const double* x = g.A + blockIdx.z * g.sA + (long long)min((int)blockIdx.y * DG_BM + (warp & 3) * 32 + lane, g.M - 1) * g.lda;
+    const double* B = g.B + blockIdx.z * g.sB + (BT ? c0 * g.ldb : c0);
+    const long long cs = BT ? g.ldb : 1, ks = BT ? 1 : g.ldb;
+    double s[8] = {};
+#pragma unroll 2
+    for (int k = 0; k < g.K; ++k) {
+        const double xk = x[k];
+        const double* y = B + k * ks;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c0 + c < g.N) s[c] = fma(xk, y[c * cs], s[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        if (fix >> c & 1u) st[lane * 8 + (c ^ ((lane >> 1) & 7))] = s[c];
+}
+
+// Entries of the warp's joined block that its fixed point is too coarse for
+// (`fix`: a bit per column of this lane's row), summed as they stand into the
+// staged block: a few by the whole warp, one after the other, more of them a row
+// a lane.
+template <bool BT>
+__device__ __noinline__ void plain_entries(const DgArgs& a, int col, uint32_t fix, double* st)
+{
+    const GemmArgs<double>& g = a.g;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (__reduce_add_sync(0xffffffffu, __popc(fix)) > 8) {
+        plain_block<BT>(a, col, st, fix);
+        return;
+    }
+    const int r0 = blockIdx.y * DG_BM + (warp & 3) * 32;
+    const int c0 = blockIdx.x * a.per * DG_BN + (warp >> 2) * 8 + col;
+    const double* A = g.A + blockIdx.z * g.sA;
+    const double* B = g.B + blockIdx.z * g.sB + (BT ? c0 * g.ldb : c0);
+    const long long cs = BT ? g.ldb : 1, ks = BT ? 1 : g.ldb;
+    for (int c = 0; c < 8; ++c)
+        for (uint32_t m = __ballot_sync(0xffffffffu, fix >> c & 1u); m; m &= m - 1) {
+            const int r = __ffs((int)m) - 1;   // inside M and N: its row and column are not zero
+            const double* x = A + (long long)(r0 + r) * g.lda;
+            const double* y = B + c * cs;
+            double s = 0.0;
+            for (int k = lane; k < g.K; k += 32) s = fma(x[k], y[k * ks], s);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) st[r * 8 + (c ^ ((r >> 1) & 7))] = s;
+        }
+}
+
+// The CTA's tiles as plain FP64 sums: columns across the lanes, eight rows a warp.
+// Bound by the FP64 pipe's two multiply-adds a clock (eight of a warp per load of
+// B).
+__device__ __noinline__ void plain_tiles(const DgArgs& a)
+{
+    const GemmArgs<double>& g = a.g;
+    const int box = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r0 = blockIdx.y * DG_BM + warp * (DG_BM / DG_WARPS);
+    const double* A = g.A + box * g.sA;
+    const double* B = g.B + box * g.sB;
+    double* O = g.O + box * g.sO;
+    if (r0 >= g.M) return;
+    for (int t = blockIdx.x * a.per; t < min((int)(blockIdx.x + 1) * a.per, a.tiles_n); ++t) {
+        const int c = t * DG_BN + lane;
+        if (c >= g.N) continue;
+        double s[DG_BM / DG_WARPS] = {};
+#pragma unroll 4
+        for (int k = 0; k < g.K; ++k) {
+            const double y = B[k * g.ldb + c];
+#pragma unroll
+            for (int u = 0; u < DG_BM / DG_WARPS; ++u)
+                s[u] = fma(A[(long long)min(r0 + u, g.M - 1) * g.lda + k], y, s[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < DG_BM / DG_WARPS; ++u) {
+            const int r = r0 + u;
+            if (r >= g.M) break;
+            double* o = O + (long long)r * g.ldo + c;
+            double src = 0.0;
+            if (g.mode == GM_ACC || (g.mode == GM_BWD && r < g.split)) src = *o;
+            else if (g.mode == GM_FWD && r >= g.split) {
+                const int pr = g.perm[box * g.sP + r];
+                src = pr >= g.split ? *o : g.W[box * g.sW + (long long)pr * g.ldw + c];
+            }
+            *o = fma(g.alpha, s[u], src);
+        }
+    }
+}
+
+// BT: B is given transposed, [n][k] with k contiguous.  CHECK: the fixed point
+// knows nothing below about 2^-58 of a row's times a column's scale (2^-51 at
+// worst, at K = 64), so an entry is taken from it only where its sum of |a||b| is
+// known to be large against that: where a factor within 2^-reach of its scale
+// meets another one (a bit per factor, joined by AND), or where nothing but zeros
+// meet.  Every other entry, and those of rows and columns with subnormals, are
+// summed as they stand on the FP64 pipe.  LU products go by their matrix instead
+// (see launch_wide).
+template <bool BT, bool CHECK>
 __global__ void __launch_bounds__(DG_THREADS, 1)
 k_digit_gemm(const __grid_constant__ DgArgs a)
 {
@@ -152,6 +257,11 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
     if (g.skip && g.skip[box]) return;
     const int t0 = blockIdx.x * a.per, cnt = min(a.per, a.tiles_n - t0);
     if (cnt <= 0) return;
+    if constexpr (!CHECK)
+        if (g.wide[box]) {
+            plain_tiles(a);
+            return;
+        }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = blockIdx.y * DG_BM;
     const uint32_t sb = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -185,6 +295,7 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
         rowsrc[tid] = s;
     }
 
+    auto expo = [](double v) { return CHECK ? exp_all(v) : exp_of(v); };
     // the block of B of one tile: column lane, k = 4 warp .. +3
     double bx[4];
     const double* Bp = BT ? B + 4 * warp + (long long)lane * g.ldb : B + (long long)(4 * warp) * g.ldb + lane;
@@ -215,10 +326,11 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
             const int rl = ps * 32 + (tid >> 4);
             int e = E_MIN;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) e = max(e, exp_of(x[ps][u]));
+            for (int u = 0; u < 4; ++u) e = max(e, expo(x[ps][u]));
 #pragma unroll
             for (int off = 8; off > 0; off >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
             if (kg == 0) rowE[rl] = e == E_BAD ? E_NAN : e;
+            if constexpr (CHECK) sp[OFF_ST + rl * 16 + kg] = reach4(x[ps], e, a.reach);   // on its way to the row's lanes
             split_to(x[ps], e, sp + rl * 128 + (((kg >> 1) ^ (rl & 7)) << 4) + ((kg & 1) << 3), A_PLANE);
         }
     }
@@ -243,6 +355,12 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
         valid |= (uint32_t)(s != -2) << u;
     }
     bool ok = true;
+    uint32_t near[4] = {}, flags = 0;   // CHECK: the bits of row `lane` of the warp's quarter, in the order of the columns'
+    if constexpr (CHECK) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            near[i] = *reinterpret_cast<const uint32_t*>(sp + OFF_ST + ((warp & 3) * 32 + lane) * 16 + 4 * (i ^ (warp >> 2)));
+    }
 
     // This lane's entries of a joined 32 x 8 block: rows 4 u + lane / 8, one
     // column.  A row that is its own source is added to in the L2 (one FP64 add
@@ -259,12 +377,19 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
 
     for (int i = 0; i <= cnt; ++i) {
         if (i < cnt) {
-            int e = max(max(exp_of(bx[0]), exp_of(bx[1])), max(exp_of(bx[2]), exp_of(bx[3])));
+            int e = max(max(expo(bx[0]), expo(bx[1])), max(expo(bx[2]), expo(bx[3])));
             atomicMax(&colE[i & 3][lane], e);
             __syncthreads();
             e = colE[i & 3][lane];
             split_to(bx, e, sp + OFF_B + (i & 1) * B_BUF + lane * 128 + (((warp >> 1) ^ (lane & 7)) << 4) + ((warp & 1) << 3),
                      B_PLANE);
+            if constexpr (CHECK) {   // into the staging buffer of each warp that joins these columns: 16 bytes a column, words swizzled
+                const unsigned char m = reach4(bx, e, a.reach);
+                const int cgi = lane >> 3;
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    sp[OFF_ST + (4 * cgi + r) * STAGE + (lane & 7) * 16 + (warp ^ (cgi << 2))] = m;
+            }
             if (warp == 0) {
                 colE[(i + 2) & 3][lane] = E_MIN;
                 colX[i & 1][lane] = e == E_BAD ? E_NAN : e - 1016;
@@ -283,6 +408,19 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
                         mma_bf16(d0 + s * DG_BN, ad + (uint64_t)(s * (A_PLANE >> 4) + kk * 2), bd + (uint64_t)(kk * 2),
                                  f16_idesc(DG_BM, DG_BN * (DG_S - s)), (kk | s) != 0);
                 mma_commit(smem_u32(&tfull[i & 1]));
+            }
+            __syncwarp();
+        }
+        // the tile's entries whose sums may be small against their scales: a bit per column of this lane's row
+        const uint32_t fix = flags;
+        flags = 0;
+        if (CHECK && i < cnt) {
+            const uint4* m = reinterpret_cast<const uint4*>(sp + OFF_ST + warp * STAGE);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint4 w = m[c];
+                const uint32_t both = (near[0] & w.x) | (near[1] & w.y) | (near[2] & w.z) | (near[3] & w.w);
+                flags |= (uint32_t)(both != 0 && (both & 0x0F0F0F0Fu) == 0) << c;
             }
             __syncwarp();
         }
@@ -328,6 +466,10 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
             }
         }
         __syncwarp();
+        if (CHECK && __any_sync(0xffffffffu, fix != 0)) {
+            plain_entries<BT>(a, j * DG_BN, fix, st);
+            __syncwarp();
+        }
         {
             double* p = Or + (long long)(t0 + j) * DG_BN;
             auto joined = [&](int u) {
@@ -380,9 +522,14 @@ void launch_digit_gemm(const GemmArgs<double>& in, bool b_transposed, int nbox, 
 {
     GemmArgs<double> g = in;
     if (g.M <= 0 || g.N <= 0 || nbox <= 0) return;
-    auto kern = b_transposed ? k_digit_gemm<true> : k_digit_gemm<false>;
+    auto kern = b_transposed ? k_digit_gemm<true, true> : g.wide ? k_digit_gemm<false, false> : k_digit_gemm<false, true>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DG_SMEM);
     DgArgs a;
+    // A product by itself (B transposed: factors given by the caller) is held to
+    // the K 2^-53 sum |a||b| of an FP64 sum: the fixed point is off by at most
+    // K 2^-57 of the scales' product, which is that where the sum is 2^-4 of it.
+    // Products with interface factors keep 29 bits of every entry (36 typically).
+    a.reach = b_transposed ? 2 : 11;
     a.tiles_n = (g.N + DG_BN - 1) / DG_BN;
     const int tiles_m = (g.M + DG_BM - 1) / DG_BM;
     // Columns of a strip are shared out so that the CTAs fill the SMs evenly: a

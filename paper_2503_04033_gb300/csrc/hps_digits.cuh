@@ -11,12 +11,28 @@ namespace hps {
 namespace {
 
 constexpr int DG_S = 8;      // digits of an operand
-constexpr int E_MIN = 1;     // scale exponent of a row or column of zeros (subnormal entries count as zero)
-constexpr int E_BAD = 2047;  // an infinity or NaN in the row or column: its scale is then kept as E_NAN
+constexpr int E_MIN = 1;     // scale exponent of a row or column of zeros (exp_of: subnormal entries count as zero)
+constexpr int E_BAD = 2047;  // an infinity or NaN (exp_all: or a subnormal) in the row or column: its scale is then kept as E_NAN
 constexpr int E_NAN = 1 << 20;
 
 __device__ __forceinline__ int exp_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ int exp_all(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x);
+    return exp_of(x) == 0 && ((hi << 1) | (uint32_t)__double2loint(x)) != 0 ? E_BAD : exp_of(x);
+}
 
+// Bits 0 .. 3: the entry is within 2^-reach of the scale; 4 .. 7: it is not zero.
+__device__ __forceinline__ unsigned char reach4(const double (&x)[4], int E, int reach)
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int e = (int)(((uint32_t)__double2hiint(x[u]) >> 20) & 0x7ffu);
+        m |= (uint32_t)(e >= max(E - reach, 1)) << u | (uint32_t)(e != 0) << (4 + u);
+    }
+    return (unsigned char)m;
+}
 // Digits of four entries under the scale exponent E: digit s of entries 0, 1
 // as FP16 pairs in d[s][0], of entries 2, 3 in d[s][1].
 __device__ __forceinline__ void split4(const double (&x)[4], int E, uint32_t (&d)[DG_S][2])
@@ -60,8 +76,8 @@ __device__ __forceinline__ void split4(const double (&x)[4], int E, uint32_t (&d
 
 // V 2^-57 of the scales, rounded once to FP64.  E: biased exponents of the two
 // scales, less 1016 (a unit of 2^-(57 + j) takes j more off).  eb_out outside
-// 0 .. 2045 asks for finish_odd: a result outside the normal range, or of a row
-// or column with an infinity or NaN.  No branch, so that several overlap.
+// 0 .. 2045 asks for a plain sum instead: a result outside the normal range, or
+// of a row or column of scale E_NAN.  No branch, so that several overlap.
 __device__ __forceinline__ double round_fixed(long long V, int E, int& eb_out)
 {
     const int sm = (int)(V >> 63);
@@ -75,15 +91,6 @@ __device__ __forceinline__ double round_fixed(long long V, int E, int& eb_out)
     const bool zero = lz == 64 && E < (1 << 19);
     eb_out = zero ? 0 : lz == 64 ? 4096 : eb;
     return __longlong_as_double(zero ? 0ll : (long long)r);
-}
-
-// The rare results: `r` has the sign, E and eb are those of its join.
-__device__ __noinline__ double finish_odd(double r, int E, int eb)
-{
-    if ((unsigned)eb <= 2045u) return r;
-    if (E >= (1 << 19)) return __longlong_as_double(0x7FF8000000000000ll);   // an infinity or NaN went in
-    const long long sg = __double_as_longlong(r) & (long long)0x8000000000000000ull;
-    return __longlong_as_double(sg | (eb < 0 ? 0ll : 0x7FF0000000000000ll));
 }
 
 }  // namespace

@@ -476,11 +476,14 @@ void if_product(int nn, int Mr, int N, int K, const MT* A, long long lda, long l
                   (double)nn * ((double)Mr * K * sizeof(MT) + 8.0 * (double)Mr * N));
 }
 
-// Merged maps of a level in the factorisation: Tn += E S (E [e][s], S [s][e]).
+// Merged maps of a level in the factorisation: Tn += E S (E [e][s], S [s][e]);
+// wide: that of the separators' LU.
 template <typename MT>
-void if_merge_product(int nn, int e, int s, const MT* E, const MT* S, MT* Tn, cudaStream_t st)
+void if_merge_product(int nn, int e, int s, const MT* E, const MT* S, MT* Tn, const int* wide,
+                      cudaStream_t st)
 {
     hps::GemmArgs<MT> a{};
+    a.wide = wide;
     a.A = E; a.lda = s; a.sA = (long long)e * s;
     a.B = S; a.ldb = e; a.sB = (long long)s * e;
     a.O = Tn; a.ldo = e; a.sO = (long long)e * e;
@@ -631,7 +634,7 @@ hps_status factor_level(IfLevel& L, int qq, void** ws, size_t* ws_bytes, int** d
     // 3 to 20 times further from 64 bits, the accumulators being cut, not rounded
     if (e > 0)
         if_merge_product<MT>(L.nn, e, s, static_cast<const MT*>(L.E), static_cast<const MT*>(L.S),
-                             static_cast<MT*>(L.Tn), st);
+                             static_cast<MT*>(L.Tn), w.wide, st);
     if (cudaGetLastError() != cudaSuccess) return HPS_ECUDA;
     std::vector<int> hs(L.nn);
     if (cudaMemcpyAsync(hs.data(), *d_status, sizeof(int) * L.nn, cudaMemcpyDeviceToHost, st) != cudaSuccess ||

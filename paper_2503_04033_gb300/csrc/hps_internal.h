@@ -109,12 +109,29 @@ struct GemmArgs {
     const T* W; long long ldw, sW;   // GM_FWD: saved rows of the panel
     const int* skip;                 // per box: nonzero = leave untouched
     int* status;                     // per box: HPS_ETIMEOUT when a bounded wait gave up (may be NULL)
+    const int* wide;                 // FP64: per box, nonzero = plain FP64 sums (NULL: the product looks at each entry)
 };
+
+// FP64 LUs run from exact digits (hps_digit.cu), which are as good as FP64 sums
+// relative to the largest entries of a row and a column of a product.  A matrix
+// whose scales lie far apart needs its small entries too, and its LU runs on
+// plain sums: launch_wide sets wide[box] where the rows' largest entries lie 2^9
+// or more apart, or (axis, dims: a collocation matrix of axis^dims nodes) where
+// the second differences of its axes do by more than 2^12.  Measured on S
+// against long double, digits : FP64 sums (geometric means of the norms of the
+// errors): rows 2^7 apart, as in every smooth, rough or cross-term problem here
+// (p <= 24), 0.5 to 1; 2^10 (impedance leaves of side 1 / 64) 5; 2^13
+// (coefficients that jump by 1e8 from node to node) 1.4, 19 at worst; 2^27 20,
+// 5e4 at worst.  Sides 1 : 10 and 1 : 100 0.7, but 8 and 16 for the median entry
+// of S, and 1 : 1e6 all but three digits of the small ones.
+void launch_wide(const double* M, long long ldm, long long sM, int n, int axis, int dims, int* wide, int nbox,
+                 cudaStream_t st);
 
 // ---------------------------------------------------------------- LU plans
 
 struct Plan {
     int n = 0, r = 0, NB = 0, nsteps = 0;
+    int axis = 0, dims = 0;          // n = axis^dims collocation nodes (0: no such grid)
     long long ldm = 0;
     size_t elt = 0;                  // bytes per LU element
     bool tc = false;                 // FP32 products on the tensor cores
@@ -194,7 +211,7 @@ inline Plan make_plan(int n, int r, hps_precision prec, int nb_opt, bool use_tc,
         }
     }
     P.per_box = P.bM + P.bF + P.bB + P.bW + P.bG + P.bP + P.bX + P.bFp + P.bBp + P.bGp + P.bInv + P.bGp2 + P.bW2 + P.bKB +
-                2 * P.bRC + 2 * P.bIT + 64;
+                2 * P.bRC + 2 * P.bIT + 64;   // 64: norms, skip and wide
     return P;
 }
 
@@ -213,6 +230,7 @@ struct Work {
     float *it1, *it2;   // format 2: 1 / (power-of-two scale) of each column of the G in Gp, Gp2
     double* norms;
     int* skip;
+    int* wide;     // FP64: boxes that run on plain sums
     long long sM, sF, sB, sG, sP, sX, sFp, sBp, sGp, sRC, sIT;
 };
 
@@ -245,6 +263,7 @@ inline Work<T> carve(const Plan& P, void* base, int nbox)
     w.sIT = (long long)(P.bIT / sizeof(float));
     w.norms = reinterpret_cast<double*>(take(align_up(2 * sizeof(double), 16)));
     w.skip = reinterpret_cast<int*>(take(align_up(sizeof(int), 16)));
+    w.wide = reinterpret_cast<int*>(take(align_up(sizeof(int), 16)));
     w.sM = (long long)(P.bM / P.elt);
     w.sF = (long long)(P.bF / P.elt);
     w.sB = (long long)(P.bB / P.elt);
@@ -283,7 +302,7 @@ void launch_build_aug(const Geometry& g, double kappa, const double* kappa_box, 
 template <typename T>
 void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* perm, long long sP, T* Ftop,
                   long long ldf, long long sF, T* Btop, long long ldb, long long sB, int* status, const int* skip,
-                  int nbox, cudaStream_t st);
+                  const int* wide, int nbox, cudaStream_t st);
 
 template <typename T>
 void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c0, int ncols,

@@ -148,6 +148,8 @@ hps_status hps_leaf2d_solve(int p, const double h[2], double kappa, int nbox, co
             }
     }
     hps::Plan PL = hps::make_plan(n, m + nrhs, HPS_FP64, 0, false, false);
+    PL.axis = p - 2;
+    PL.dims = 2;
     const size_t tab_bytes = hps::align_up(sizeof(double) * (size_t)ntab, 256);
     const size_t st_bytes = hps::align_up(sizeof(int) * (size_t)nbox, 256);
     const size_t bytes = tab_bytes + st_bytes + PL.per_box * (size_t)nbox;

@@ -72,7 +72,9 @@ extern "C" hps_status hps_leaf_build_dtn_noalloc(const hps_leaf_kind* kind, int 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
     // Scratch layout: [D | D2 | status words | per-box LU workspace x chunk].
-    const Plan P = make_plan(n, m, HPS_FP64, 0, false, false);
+    Plan P = make_plan(n, m, HPS_FP64, 0, false, false);
+    P.axis = p - 2;
+    P.dims = 3;
     const size_t tables = align_up(2 * 3 * (size_t)pp * sizeof(double), 256);
     const size_t fixed = tables + (box_status ? 0 : align_up((size_t)nbox * sizeof(int), 256));
     if (p > kMaxNoallocP || fixed + P.per_box > kScratchBytes) return HPS_ENOMEM;   // one box does not fit

@@ -10,7 +10,8 @@
 //      hand their entries over, the block's unit triangle (its inverse, kept)
 //      turns them into rows of U, and every other row subtracts its stored
 //      multipliers times them (16 multiply-adds per value read back; FP64 as
-//      digit products on the tensor cores, see hps_digits.cuh);
+//      digit products on the tensor cores, see hps_digits.cuh, except in boxes
+//      whose scales lie too far apart for them);
 //   2. factor the block: per column every warp offers its largest candidate
 //      with its row, the CTA picks one after one barrier (in a cluster the
 //      CTAs' offers are exchanged through distributed shared memory and a
@@ -259,7 +260,18 @@ struct PanelArgs {
     long long sP;
     int* status;
     const int* skip;
+    const int* wide;   // FP64: boxes whose left products run as plain sums (see launch_wide)
 };
+
+// Entry (row, column) of the product of an earlier block's multipliers with u as
+// an FP64 sum; l, u: the first multiplier and value, a step apart each.
+template <int IB>
+__device__ __noinline__ double plain_entry(const double* l, long long step, const double* u)
+{
+    double s = 0.0;
+    for (int k = 0; k < IB; ++k) s = fma(l[k * step], u[k * IB], s);
+    return s;
+}
 
 // Shared memory of a panel CTA.
 template <typename T, int IB>
@@ -305,6 +317,8 @@ k_panel(const PanelArgs<T> a)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R0 = a.n - a.k;
     T* P = a.M + box * a.sM + (long long)a.k * a.ldm + a.k;   // the panel's corner
+    bool hard = false;   // FP64: left products as plain sums
+    if constexpr (sizeof(T) == 8) hard = a.wide[box] != 0;
     auto row_of = [&](int rr) { return ((rr * PW + warp) * C + rank) * 32 + lane; };
     // the warp's row groups that exist (all of a group's lanes may still be past the last row)
     const int nrr = min(RPT, max(0, ((R0 + 31) / 32 - rank - warp * C + PW * C - 1) / (PW * C)));
@@ -427,7 +441,7 @@ k_panel(const PanelArgs<T> a)
                 // (K = IB <= 16: every accumulator stays below 2^21); as 16 multiply-adds
                 // per entry on the FP64 pipe, 64 clocks a warp each, it took seven times as long
                 const int g = lane >> 2, q = lane & 3;
-                if (warp < IB / 8) {
+                if (warp < IB / 8 && !hard) {
                     double v[4];
                     int ex = E_MIN;
 #pragma unroll
@@ -445,6 +459,20 @@ k_panel(const PanelArgs<T> a)
                     if (q == 0) s.ue[8 * warp + g] = ex == E_BAD ? E_NAN : ex - 1018;
                 }
                 __syncthreads();
+                if (hard) {
+#pragma unroll 1
+                    for (int kk = 0; kk < IB; ++kk)
+#pragma unroll
+                        for (int rr = 0; rr < RPT; ++rr) {
+                            const bool on = pidx[rr] == -1 || pidx[rr] >= je + IB;
+                            const T l = on ? Lt[(long long)(je + kk) * R0 + row_of(rr)] : T(0);
+                            if (on) {
+#pragma unroll
+                                for (int c = 0; c < IB; ++c) x[rr][c] -= l * s.u[kk][c];
+                            }
+                        }
+                    continue;
+                }
 #pragma unroll
                 for (int rr = 0; rr < RPT; ++rr) {
                     if (rr >= nrr) continue;
@@ -507,8 +535,11 @@ k_panel(const PanelArgs<T> a)
                                 double2 r;
                                 r.x = round_fixed(V[2 * h], ea[h] + ue.x, eb0);
                                 r.y = round_fixed(V[2 * h + 1], ea[h] + ue.y, eb1);
-                                if ((unsigned)eb0 > 2045u) r.x = finish_odd(r.x, ea[h] + ue.x, eb0);
-                                if ((unsigned)eb1 > 2045u) r.y = finish_odd(r.y, ea[h] + ue.y, eb1);
+                                if (((unsigned)eb0 > 2045u || (unsigned)eb1 > 2045u) && (onm >> (16 * mt + 8 * h + g) & 1)) {
+                                    const double* l = Lt + (long long)je * R0 + row0 + 16 * mt + 8 * h + g;
+                                    if ((unsigned)eb0 > 2045u) r.x = plain_entry<IB>(l, R0, &s.u[0][8 * nt + 2 * q]);
+                                    if ((unsigned)eb1 > 2045u) r.y = plain_entry<IB>(l, R0, &s.u[0][8 * nt + 2 * q + 1]);
+                                }
                                 *tile_row(tile, 16 * mt + 8 * h + g, 4 * nt + q) = r;
                             }
                         }
@@ -894,7 +925,7 @@ size_t panel_smem(int ib, int nb)
 template <typename T>
 void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* perm, long long sP, T* Ftop,
                   long long ldf, long long sF, T* Btop, long long ldb, long long sB, int* status, const int* skip,
-                  int nbox, cudaStream_t st)
+                  const int* wide, int nbox, cudaStream_t st)
 {
     static const bool once = [] {
         for (int i = 0; i < 4; ++i)
@@ -937,7 +968,7 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
     // multiple of 8 and k one of 16 (make_plan rounds every stride up, steps are
     // NB wide).  The multipliers' scratch is the step's F block, which the inverse and the
     // product after this overwrite
-    PanelArgs<T> a{M, ldm, sM, n, k, nb, Ftop, sF, perm, sP, status, skip};
+    PanelArgs<T> a{M, ldm, sM, n, k, nb, Ftop, sF, perm, sP, status, skip, wide};
     prof_begin(KC_PANEL, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nbox * bc));
@@ -960,8 +991,8 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
 }
 
 template void launch_panel<float>(float*, long long, long long, int, int, int, int*, long long, float*, long long,
-                                  long long, float*, long long, long long, int*, const int*, int, cudaStream_t);
+                                  long long, float*, long long, long long, int*, const int*, const int*, int, cudaStream_t);
 template void launch_panel<double>(double*, long long, long long, int, int, int, int*, long long, double*, long long,
-                                   long long, double*, long long, long long, int*, const int*, int, cudaStream_t);
+                                   long long, double*, long long, long long, int*, const int*, const int*, int, cudaStream_t);
 
 }  // namespace hps
