@@ -49,11 +49,15 @@ __global__ void k_iti_tables(const ItiTables a, double* D, double* D2)
 // interior rows (Eq. 2: -sum D2 along the three grid lines - kappa^2 b), then
 // the m face rows (outward normal derivative along the face's axis); the
 // columns of a half are the n interior then m face unknowns.  D and D2 are
-// [3][p][p] (axis-major), b [nbox][p^3].
+// [3][p][p] (axis-major), b [nbox][p^3].  The face rows of axis a, of order
+// 1 / h_a, are written times scale[a], the power of two that brings them to the
+// interior rows' order 1 / h^2: the LU's products share a scale per row and
+// column (see launch_wide), and with the rows as they come R was 5 (side 1 / 64) to
+// 1000 times (1 / 1024) further from long double than on FP64 sums.
 __global__ void __launch_bounds__(256)
 k_build_iti(int p, int n, int m, const double* __restrict__ D, const double* __restrict__ D2, double kappa2,
-            double eta, const double* __restrict__ b, int nrhs, const double* __restrict__ f, double* __restrict__ M,
-            long long ldm, long long sM, int* status)
+            double eta, const double3 scale, const double* __restrict__ b, int nrhs, const double* __restrict__ f,
+            double* __restrict__ M, long long ldm, long long sM, int* status)
 {
     const int box = blockIdx.y;
     const int N = n + m, N2 = 2 * N;
@@ -113,7 +117,8 @@ k_build_iti(int p, int n, int m, const double* __restrict__ D, const double* __r
         } else {
             const int r = lr - n, f = r / qq, s = r - f * qq, axis = f >> 1;
             const int a = s % q + 1, c = s / q + 1, e = (f & 1) ? p - 1 : 0;
-            const double sg = (f & 1) ? 1.0 : -1.0;
+            const double sc = axis == 0 ? scale.x : axis == 1 ? scale.y : scale.z;
+            const double sg = (f & 1) ? sc : -sc;
             for (int l = threadIdx.x; l < p; l += blockDim.x) {
                 int ii, jj, kk;
                 if (axis == 0) { ii = l; jj = a; kk = c; }
@@ -124,10 +129,10 @@ k_build_iti(int p, int n, int m, const double* __restrict__ D, const double* __r
             if (threadIdx.x == 0) {
                 // the impedance coupling between the halves, and F
                 if (half == 0) {
-                    row[N + n + r] = -eta;
-                    row[N2 + r] = 1.0;
+                    row[N + n + r] = -eta * sc;
+                    row[N2 + r] = sc;
                 } else {
-                    row[n + r] = eta;
+                    row[n + r] = eta * sc;
                 }
             }
         }
@@ -261,6 +266,14 @@ hps_status hps_leaf_iti_solve(const hps_leaf_kind* kind, double eta, int nbox, c
     ta.p = p;
     for (int a = 0; a < 3; ++a) ta.h[a] = kind->h[a];
     hps::cheb_diff(p, ta.Dhat);
+    double d2 = 0.0;   // second derivative at the first interior node, its largest entry
+    for (int l = 0; l < p; ++l) d2 += ta.Dhat[p + l] * ta.Dhat[l * p + 1];
+    const double inner = 4.0 * std::fabs(d2) / std::pow(std::min({ta.h[0], ta.h[1], ta.h[2]}), 2);
+    auto pow2 = [&](double h) {   // 1 where the sides leave the range of FP64
+        const double e = std::round(std::log2(inner * h / (2.0 * std::fabs(ta.Dhat[0]))));
+        return std::fabs(e) < 400.0 ? std::exp2(e) : 1.0;
+    };
+    const double3 scale = make_double3(pow2(ta.h[0]), pow2(ta.h[1]), pow2(ta.h[2]));
     hps::Plan PL = hps::make_plan(N2, m + nrhs, HPS_FP64, 0, false, false);
     const size_t tab_bytes = hps::align_up(sizeof(double) * 6 * pp, 256);
     const size_t st_bytes = hps::align_up(sizeof(int) * (size_t)nbox, 256);
@@ -276,7 +289,7 @@ hps_status hps_leaf_iti_solve(const hps_leaf_kind* kind, double eta, int nbox, c
     if (cudaMemsetAsync(status, 0, sizeof(int) * (size_t)nbox, st) != cudaSuccess) rc = HPS_ECUDA;
     if (rc == HPS_OK) {
         k_build_iti<<<dim3((unsigned)((N2 + kItiRows - 1) / kItiRows), (unsigned)nbox), 256, 0, st>>>(
-            p, n, m, dtab, dtab + 3 * pp, kind->kappa * kind->kappa, eta, b, nrhs, f, w.M, PL.ldm, w.sM, status);
+            p, n, m, dtab, dtab + 3 * pp, kind->kappa * kind->kappa, eta, scale, b, nrhs, f, w.M, PL.ldm, w.sM, status);
         hps::lu_factor<double>(PL, w, nbox, status, st);
         hps::lu_backward<double>(PL, w, nbox, N2, m + nrhs, nullptr, st);
         const long long mm = (long long)m * m, nm = (long long)n * m;
