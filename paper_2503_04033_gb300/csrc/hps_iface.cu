@@ -326,6 +326,29 @@ __global__ void k_if_down(const IfDesc* __restrict__ desc, const int* __restrict
     }
 }
 
+// Sums over the lanes of V values each (V a power of two up to 32): lane l ends
+// with the sum of value l / (32 / V) in s[0].  Halves are exchanged, so that V
+// values take V - 1 adds and as many shuffles before one value is left, not 5 V.
+// The order of the additions is that of a butterfly.
+template <int V>
+__device__ __forceinline__ void lane_sums(double (&s)[V], int lane)
+{
+#pragma unroll
+    for (int st = 0; st < 5; ++st) {
+        const int o = 16 >> st, half = V >> (st + 1);
+        if (half > 0) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < half; ++i) {
+                const double give = up ? s[i] : s[i + half], keep = up ? s[i + half] : s[i];
+                s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        } else {
+            s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+        }
+    }
+}
+
 // O = [acc] O + alpha A B for a batch of small-N products (N = nrhs <= 16,
 // NC columns per pass), A in the storage type MT, B and O in FP64, sums in
 // FP64.  A warp takes four rows of A and reads 16 bytes of each per lane and
@@ -335,18 +358,22 @@ __global__ void k_if_down(const IfDesc* __restrict__ desc, const int* __restrict
 // integer pipe: the FP64 pipe, two multiply-adds per clock and SM, then has
 // one per entry and load, which bounds FP32 matrices at 2.5 TB/s (FP64 ones at
 // HBM).  A refined solve of 8 x 8 x 8 boxes at p = 12 (six sweeps): 56 -> 20 ms
-// against a thread group per row with the entries converted on the FP64 pipe.  A [M][K] (pitch lda); B element (k, c) at k bk + c bc; O element
-// (r, c) at r ok + c oc.  VEC: the rows of A start on 16 bytes.
-template <int NC, typename MT, bool VEC>
+// against a thread group per row with the entries converted on the FP64 pipe.
+// A [M][K] (pitch lda); B element (k, c) at k bk + c bc; O element (r, c) at
+// r ok + c oc.  VEC: the rows of A start on 16 bytes.  RW = 1: a warp takes one
+// row, a lane an entry: levels of few rows, whose four-row warps left most SMs
+// idle and most lanes of the others (K = 36 is nine lanes of four entries).
+template <int NC, typename MT, int RW, bool VEC>
 __global__ void __launch_bounds__(256) k_if_mv(int Mr, int K, int N, int KS, const MT* __restrict__ A, long long lda,
                                                long long sA, const double* __restrict__ B, long long sB,
                                                long long bk, long long bc, double* __restrict__ O, long long sO,
                                                long long ok, long long oc, double alpha, int acc,
                                                const int* __restrict__ skip)
 {
-    constexpr int RW = 4, U = 16 / sizeof(MT);   // rows of a warp, entries of a 16-byte load
+    constexpr int U = RW == 1 ? 1 : 16 / (int)sizeof(MT);   // entries of a lane and step
     if (skip && *skip) return;
-    __shared__ double red[8][RW][NC];
+    constexpr int V = RW * NC;   // sums of a warp
+    __shared__ double red[8][V];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = warp / KS, part = warp - grp * KS;
     const int row0 = (blockIdx.x * (8 / KS) + grp) * RW;
@@ -357,11 +384,9 @@ __global__ void __launch_bounds__(256) k_if_mv(int Mr, int K, int N, int KS, con
 #pragma unroll
     for (int r = 0; r < RW; ++r) Ar[r] = Ab + (long long)min(row0 + r, Mr - 1) * lda;
     for (int c0 = 0; c0 < N; c0 += NC) {
-        double s[RW][NC];
+        double s[V];
 #pragma unroll
-        for (int r = 0; r < RW; ++r)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) s[r][c] = 0.0;
+        for (int i = 0; i < V; ++i) s[i] = 0.0;
         if (row0 < Mr) {
 #pragma unroll 2
             for (int k = (part * 32 + lane) * U; k < K; k += KS * 32 * U) {
@@ -393,31 +418,28 @@ __global__ void __launch_bounds__(256) k_if_mv(int Mr, int K, int N, int KS, con
                         else a = av[r][u];
 #pragma unroll
                         for (int c = 0; c < NC; ++c)
-                            if (c0 + c < N) s[r][c] += a * bv[u][c];
+                            if (c0 + c < N) s[r * NC + c] += a * bv[u][c];
                     }
             }
         }
-#pragma unroll
-        for (int r = 0; r < RW; ++r)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s[r][c] += __shfl_xor_sync(0xffffffffu, s[r][c], o);
-                if (lane == 0) red[warp][r][c] = s[r][c];
-            }
-        if (KS > 1) __syncthreads();
-        else __syncwarp();
-        if (part == 0 && lane < RW * NC) {
-            const int r = lane / NC, c = lane - r * NC;
-            if (row0 + r < Mr && c0 + c < N) {
-                double v = 0.0;
-                for (int w = 0; w < KS; ++w) v += red[warp + w][r][c];
-                double* o = Ob + (long long)(row0 + r) * ok + (long long)(c0 + c) * oc;
-                *o = (acc ? *o : 0.0) + alpha * v;
+        lane_sums<V>(s, lane);
+        const int i = lane / (32 / V);
+        const bool first = lane % (32 / V) == 0;
+        double v = s[0];
+        if (KS > 1) {
+            if (first) red[warp][i] = v;
+            __syncthreads();
+            if (part == 0) {
+                v = 0.0;
+                for (int w = 0; w < KS; ++w) v += red[warp + w][i];
             }
         }
+        const int r = i / NC, c = i - r * NC;
+        if (part == 0 && first && row0 + r < Mr && c0 + c < N) {
+            double* o = Ob + (long long)(row0 + r) * ok + (long long)(c0 + c) * oc;
+            *o = (acc ? *o : 0.0) + alpha * v;
+        }
         if (KS > 1) __syncthreads();
-        else __syncwarp();
     }
 }
 
@@ -426,17 +448,18 @@ void launch_mv(int nn, int Mr, int N, int K, const MT* A, long long lda, long lo
                long long bk, long long bc, double* O, long long sO, long long ok, long long oc, double alpha, int acc,
                const int* skip, cudaStream_t st)
 {
-    // Warps per row group: more while the level's rows leave SMs without eight
-    // CTAs' worth of warps and every warp still has a step of K.
+    // A row a warp where four would leave SMs without a CTA.  Warps per row group:
+    // more while the level's rows leave SMs without eight CTAs' worth of warps and
+    // every warp still has a step of K.
+    const bool few = (long long)nn * Mr <= 152LL * 32;
+    const int rw = few ? 1 : 4, step = few ? 32 : 32 * (int)(16 / sizeof(MT));
     int ks = 1;
-    while (ks < 8 && (long long)nn * Mr * ks < 152LL * 8 * 32 && K > ks * 32 * (int)(16 / sizeof(MT))) ks *= 2;
-    const int rows_per_cta = 32 / ks;
+    while (ks < 8 && (long long)nn * Mr * ks < 152LL * 8 * 8 * rw && K > ks * step) ks *= 2;
+    const int rows_per_cta = 8 * rw / ks;
     const bool vec = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && lda * sizeof(MT) % 16 == 0 && sA * sizeof(MT) % 16 == 0;
     const dim3 grd((unsigned)((Mr + rows_per_cta - 1) / rows_per_cta), (unsigned)nn);
-    if (vec)
-        k_if_mv<NC, MT, true><<<grd, 256, 0, st>>>(Mr, K, N, ks, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip);
-    else
-        k_if_mv<NC, MT, false><<<grd, 256, 0, st>>>(Mr, K, N, ks, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip);
+    auto kern = few ? k_if_mv<NC, MT, 1, false> : vec ? k_if_mv<NC, MT, 4, true> : k_if_mv<NC, MT, 4, false>;
+    kern<<<grd, 256, 0, st>>>(Mr, K, N, ks, A, lda, sA, B, sB, bk, bc, O, sO, ok, oc, alpha, acc, skip);
 }
 
 template <typename MT>
