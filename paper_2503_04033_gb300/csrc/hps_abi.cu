@@ -584,10 +584,11 @@ hps_status refine_chunk(hps_ctx* ctx, const Geometry& g, const CallSpec& cs, con
         } else
             launch_residual(g, cs.kappa, cs.kappa_dev, nbox, b, p3, cs.rhs_kind, cs.r, cs.rhs, cs.s_rhs, X, ldx, sX,
                             w.M + g.n, P.ldm, w.sM, w.skip, st, w.kb, cs.beta);
-        if (narrow_solve(P, w, nbox, g.n, cs.r, w.skip, st)) {
-        } else if (P.tc) {
-            if (!tc_lu_forward(P, w, nbox, g.n, cs.r, w.skip, st)) return HPS_ECUDA;
-            if (!tc_lu_backward(P, w, nbox, g.n, cs.r, w.skip, st)) return HPS_ECUDA;
+        if (P.tc) {
+            if (!narrow_solve(P, w, nbox, g.n, cs.r, w.skip, st)) {
+                if (!tc_lu_forward(P, w, nbox, g.n, cs.r, w.skip, st)) return HPS_ECUDA;
+                if (!tc_lu_backward(P, w, nbox, g.n, cs.r, w.skip, st)) return HPS_ECUDA;
+            }
         } else {
             lu_forward<float>(P, w, nbox, g.n, cs.r, w.skip, st);
             lu_backward<float>(P, w, nbox, g.n, cs.r, w.skip, st);

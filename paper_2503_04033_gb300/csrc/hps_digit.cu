@@ -504,18 +504,6 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-int sm_count()
-{
-    static int n = 0;   // the library serves one kind of GPU; 152 on GB300
-    if (!n) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            n = 152;
-    }
-    return n;
-}
-
 }  // namespace
 
 void launch_digit_gemm(const GemmArgs<double>& in, bool b_transposed, int nbox, cudaStream_t st)

@@ -81,7 +81,8 @@ struct IfLevel {
     double* y = nullptr;      // solve: W^{-1} (h^a_3 + h^b_3) [nn][s_pad][nrhs]
 };
 
-constexpr int kMaxSeparator = 14000;   // a panel's cluster holds 16,384 rows
+constexpr int kMaxSeparator = 14000;
+static_assert(kMaxSeparator <= hps::kPanelMaxRows, "a separator's LU starts with a panel of all its rows");
 constexpr int kRefineMax = 10;         // FP32_IR: most corrections per solve
 constexpr double kRefineTol = 1e-14;   // FP32_IR: stop when ||du|| <= tol ||u||
 
@@ -451,10 +452,11 @@ void launch_mv(int nn, int Mr, int N, int K, const MT* A, long long lda, long lo
     // A row a warp where four would leave SMs without a CTA.  Warps per row group:
     // more while the level's rows leave SMs without eight CTAs' worth of warps and
     // every warp still has a step of K.
-    const bool few = (long long)nn * Mr <= 152LL * 32;
+    const long long sms = hps::sm_count();
+    const bool few = (long long)nn * Mr <= sms * 32;
     const int rw = few ? 1 : 4, step = few ? 32 : 32 * (int)(16 / sizeof(MT));
     int ks = 1;
-    while (ks < 8 && (long long)nn * Mr * ks < 152LL * 8 * 8 * rw && K > ks * step) ks *= 2;
+    while (ks < 8 && (long long)nn * Mr * ks < sms * 8 * 8 * rw && K > ks * step) ks *= 2;
     const int rows_per_cta = 8 * rw / ks;
     const bool vec = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && lda * sizeof(MT) % 16 == 0 && sA * sizeof(MT) % 16 == 0;
     const dim3 grd((unsigned)((Mr + rows_per_cta - 1) / rows_per_cta), (unsigned)nn);

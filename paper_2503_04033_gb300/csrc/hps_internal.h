@@ -14,12 +14,29 @@ namespace hps {
 
 constexpr int kMaxP = 24;
 constexpr int kMaxNB = 128;          // largest LU block (K of every update product)
+constexpr int kPanelMaxRows = 16384; // rows of a panel: 8 CTAs of 256 threads with eight rows each
+static_assert((kMaxP - 2) * (kMaxP - 2) * (kMaxP - 2) <= kPanelMaxRows, "a leaf's LU starts with a panel of all its rows");
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 enum RhsKind { RHS_DTN = 0, RHS_LOAD = 1, RHS_TRACE = 2, RHS_DTN_LOAD = 3 };
 
-// Update-product epilogue modes (see gemm description in hps_kernels.cuh).
+// SMs of the GPU (152 on GB300); every device of the process is of one kind.
+inline int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+            v = 152;
+        return v;
+    }();
+    return n;
+}
+
+// Where an update product O = src + alpha A B takes its source row r: SET nothing,
+// ACC O's row, FWD nothing above `split` and below it O's row or, where perm[r] <
+// split, row perm[r] of W, BWD O's row above `split` and nothing below.
 // GM_SRC (digit products only): src is row r of W.
 enum GemmMode { GM_SET = 0, GM_ACC = 1, GM_FWD = 2, GM_BWD = 3, GM_SRC = 4 };
 

@@ -28,6 +28,7 @@
 namespace {
 
 constexpr int kItiMaxP = 16;
+static_assert(2 * (kItiMaxP - 2) * (kItiMaxP - 2) * (kItiMaxP + 4) <= hps::kPanelMaxRows, "the LU's first panel holds 2 (n + m) rows");
 constexpr int kItiRows = 4;   // rows per CTA of the build
 
 // The reference Chebyshev matrix and the box size by value: the D and D2

@@ -32,6 +32,7 @@
 // that form: 128 columns of 1000 rows 475 -> 217 us (one box) and 1.94 -> 0.92 ms
 // (512 boxes); 64 FP64 columns of 216 rows 660 -> 160 us.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <type_traits>
 
@@ -297,6 +298,7 @@ struct PanelSmem {
     int sing;
 };
 static_assert(PW == 8 && kMaxCluster == 8, "best_offer compares eight");
+static_assert(PT * 8 * kMaxCluster == kPanelMaxRows, "the largest shape below");
 
 // CTAs per SM by the registers of a thread's rows: two of up to 64 (FP32) or 32 (FP64, whose products take 90 more).
 template <typename T>
@@ -920,6 +922,31 @@ size_t panel_smem(int ib, int nb)
     return align_up(head, 16) + ldl * ldl * sizeof(T);
 }
 
+
+// Shared-memory limits of the kernels, a property of a kernel on a device: raised
+// when a device runs its first panel.
+template <typename T>
+void panel_attributes()
+{
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_relaxed) & bit) return;
+    const int nb = sizeof(T) == 4 ? kMaxNB : 64;
+    for (int i = 0; i < 4; ++i)
+        cudaFuncSetAttribute(panel_kernel<T>(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)panel_smem<T>(panel_shape<T>(i).ib, nb));
+    cudaFuncSetAttribute(k_tri_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * nb * nb * (int)sizeof(T));
+    done.fetch_or(bit, std::memory_order_relaxed);
+}
+
+__global__ void k_refuse(int nbox, int* status)
+{
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < nbox && status[b] == 0) status[b] = HPS_EINVAL;
+}
+
 }  // namespace
 
 template <typename T>
@@ -927,15 +954,7 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
                   long long ldf, long long sF, T* Btop, long long ldb, long long sB, int* status, const int* skip,
                   const int* wide, int nbox, cudaStream_t st)
 {
-    static const bool once = [] {
-        for (int i = 0; i < 4; ++i)
-            cudaFuncSetAttribute(panel_kernel<T>(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)panel_smem<T>(panel_shape<T>(i).ib, sizeof(T) == 4 ? kMaxNB : 64));
-        cudaFuncSetAttribute(k_tri_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * (sizeof(T) == 4 ? kMaxNB * kMaxNB : 64 * 64) * sizeof(T)));
-        return true;
-    }();
-    (void)once;
+    panel_attributes<T>();
     // Rows per thread and cluster size: the fewest waves of (chain of a pivot +
     // the elimination's issue), in clocks fitted to timings of every shape at 1
     // to 512 boxes and 64 to 5832 rows: the chain takes about 1500 alone and 2900
@@ -945,7 +964,11 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
     // by shape, 512 boxes of 2744 rows 3.6 ms with four CTAs of four rows a thread
     // against 3.9 with two of eight; FP64, 64 columns: 8 boxes of 216 rows 160 us
     // with one CTA a box against 204 with eight.
-    const int R0 = n - k;
+    const int R0 = n - k, sms = sm_count();
+    if (R0 > kPanelMaxRows) {   // every caller's matrices are smaller (static_assert): nothing is left out silently
+        k_refuse<<<(unsigned)((nbox + 255) / 256), 256, 0, st>>>(nbox, status);
+        return;
+    }
     int bi = 3, bc = kMaxCluster;
     double best = -1.0;
     for (int i = 0; i < 4; ++i) {
@@ -955,9 +978,9 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
             // blocks of 8 columns only for FP64 panels that nothing else holds, so that
             // the arithmetic does not depend on the batch
             if (sh.ib != 16 && R0 <= PT * 4 * kMaxCluster) continue;
-            const long long ctas = (long long)nbox * c, slots = 152LL * sh.occ;
+            const long long ctas = (long long)nbox * c, slots = (long long)sms * sh.occ;
             const double waves = (double)((ctas + slots - 1) / slots);
-            const double share = (double)std::min<long long>(sh.occ, (ctas + 151) / 152);
+            const double share = (double)std::min<long long>(sh.occ, (ctas + sms - 1) / sms);
             const double groups = (double)((R0 + 32 * c - 1) / (32 * c));
             const double chain = sizeof(T) == 4 ? (c == 1 ? 1500.0 : 2900.0) : (c == 1 ? 4300.0 : 6000.0);
             const double cost = waves * (chain + share * groups * sh.group) + 0.2 * c;
