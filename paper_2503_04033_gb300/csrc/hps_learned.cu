@@ -257,6 +257,26 @@ __global__ void k_split_uv(int B, int mr, const float* __restrict__ y, int ldy, 
     }
 }
 
+// T[b] = T0 + s U[b] V[b]^T as plain FP64 sums, an entry a thread; NA partial sums,
+// joined pairwise (eight beyond rank 16: they round less than one of all terms).
+template <int NA>
+__global__ void k_lowrank_plain(int m, int r, const double* __restrict__ T0, double s, const double* __restrict__ U,
+                                const double* __restrict__ V, double* __restrict__ T)
+{
+    const int i = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= m) return;
+    const long long row = (long long)blockIdx.z * m + i, col = (long long)blockIdx.z * m + j;
+    double acc[NA] = {};
+    for (int k = 0; k < r; k += NA)
+#pragma unroll
+        for (int u = 0; u < NA; ++u)
+            if (k + u < r) acc[u] = fma(U[row * r + k + u], V[col * r + k + u], acc[u]);
+#pragma unroll
+    for (int h = NA / 2; h > 0; h >>= 1)
+#pragma unroll
+        for (int u = 0; u < h; ++u) acc[u] += acc[u + h];
+    T[row * m + j] = T0[(long long)i * m + j] + s * acc[0];
+}
 
 // splitmix64 -> uniform in [-a, a)
 unsigned long long splitmix(unsigned long long& s)
@@ -674,7 +694,20 @@ hps_status hps_lowrank_dtn(int nbox, int m, int rank, const double* T0, double s
     if (nbox == 0) return HPS_OK;
     // The FP64 product U V^T from exact digits: as K = rank multiply-adds per
     // entry on the FP64 pipes it took 20.3 ms for 512 boxes of m = 600, rank 32;
-    // from digits 1.6 ms.
+    // from digits 1.8 ms.  A rank below eight pads the digits' K of 16 more than
+    // the FP64 pipes need (200 boxes of m = 600, rank 4: 625 us plain, 1245 from
+    // digits; rank 8 1118 : 901), and a digit product takes 11 us at least, which
+    // plain sums of the sizes below do not (rank 8: 16 boxes of m = 216 14.6 : 22.3
+    // us, 64 49.6 : 59.3, 700 519 : 477; rank 16, one box of m = 384 10.6 : 12.0, 600
+    // 24.8 : 12.6; rank 32, m = 216 8.3 : 11.8, 384 19.3 : 12.0).
+    const double work = (double)nbox * m * m * rank;
+    const double few = rank < 8 ? 1e300 : rank == 8 ? 3.3e7 : rank <= 16 ? 2.5e6 : rank <= 32 ? 2e6 : 1e6;
+    if (work < few && m <= 65535) {
+        auto kern = rank <= 16 ? k_lowrank_plain<1> : k_lowrank_plain<8>;
+        kern<<<dim3((unsigned)((m + 127) / 128), (unsigned)m, (unsigned)nbox), 128, 0,
+                          static_cast<cudaStream_t>(stream)>>>(m, rank, T0, scale, U, V, T);
+        return cudaGetLastError() == cudaSuccess ? HPS_OK : HPS_ECUDA;
+    }
     hps::GemmArgs<double> g{};
     g.A = U; g.lda = rank; g.sA = (long long)m * rank;
     g.B = V; g.ldb = rank; g.sB = (long long)m * rank;

@@ -37,20 +37,24 @@ def _factors(kind, m, r, rng):
 
 
 @pytest.mark.parametrize("kind", ["plain", "opposed", "opposed_mild", "spread", "few", "subnormal"])
-@pytest.mark.parametrize("m,r", [(2, 2), (33, 17), (129, 64), (160, 65)])
-def test_lowrank_entries_are_as_good_as_fp64_sums(kind, m, r):
+@pytest.mark.parametrize("m,r,nbox", [(2, 2, 1), (33, 17, 1), (33, 17, 130), (129, 64, 1), (160, 65, 1), (200, 8, 110),
+                                      (300, 7, 2)])
+def test_lowrank_entries_are_as_good_as_fp64_sums(kind, m, r, nbox):
+    """Sizes on both sides of the lines between plain sums and digits."""
     import torch
     import paper_2503_04033_gb300 as H
-    U, V = _factors(kind, m, r, np.random.default_rng(10 * m + r))
-    T = torch.full((1, m, m), np.nan, dtype=torch.float64, device="cuda")
-    H.hps_lowrank_dtn(1, m, r, torch.zeros(m, m, dtype=torch.float64, device="cuda"), 1.0,
+    rng = np.random.default_rng(10 * m + r)
+    U, V = (np.stack(x) for x in zip(*(_factors(kind, m, r, rng) for _ in range(nbox))))
+    T = torch.full((nbox, m, m), np.nan, dtype=torch.float64, device="cuda")
+    H.hps_lowrank_dtn(nbox, m, r, torch.zeros(m, m, dtype=torch.float64, device="cuda"), 1.0,
                       torch.from_numpy(U).cuda(), torch.from_numpy(V).cuda(), T)
     L = np.longdouble
-    ref = U.astype(L) @ V.astype(L).T
-    size = np.abs(U).astype(L) @ np.abs(V).astype(L).T
-    err = np.abs(T.cpu().numpy()[0].astype(L) - ref)
-    bound = (2 * min(r, 64) + 2 * ((r + 63) // 64)) * L(2.0) ** -53 * size + L(2.0) ** -1073
-    assert (err <= bound).all(), float((err / np.maximum(bound, L(1e-4000))).max())
+    for b in {0, nbox // 2, nbox - 1}:
+        ref = U[b].astype(L) @ V[b].astype(L).T
+        size = np.abs(U[b]).astype(L) @ np.abs(V[b]).astype(L).T
+        err = np.abs(T[b].cpu().numpy().astype(L) - ref)
+        bound = (2 * min(r, 64) + 2 * ((r + 63) // 64)) * L(2.0) ** -53 * size + L(2.0) ** -1073
+        assert (err <= bound).all(), float((err / np.maximum(bound, L(1e-4000))).max())
 
 
 def _lu_longdouble(A, B):
