@@ -354,7 +354,7 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
         other |= (uint32_t)(s >= 0) << u;
         valid |= (uint32_t)(s != -2) << u;
     }
-    bool ok = true;
+    int lost = -1;   // the tile whose wait gave up
     uint32_t near[4] = {}, flags = 0;   // CHECK: the bits of row `lane` of the warp's quarter, in the order of the columns'
     if constexpr (CHECK) {
 #pragma unroll
@@ -398,7 +398,7 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
             fence_proxy_async_smem();
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (tid == 0 && lost < 0) {
                 tc_fence_after();
                 const uint32_t d0 = tmem + (uint32_t)((i & 1) * 256);
                 const uint64_t ad = sw128_desc(sb), bd = sw128_desc(sb + OFF_B + (uint32_t)(i & 1) * B_BUF);
@@ -436,9 +436,9 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
 #pragma unroll
             for (int u = 0; u < 8; ++u) src[u] = in && (other >> u & 1) ? w[4 * u * g.ldw] : 0.0;
         }
-        if (ok) ok = wait(&tfull[buf], j >> 1);
+        if (lost < 0 && !wait(&tfull[buf], j >> 1)) lost = j;
         tc_fence_after();
-        const int Ea = ok ? rowE[rq + lane] : E_NAN;
+        const int Ea = lost < 0 ? rowE[rq + lane] : E_NAN;
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {
             uint32_t v[DG_S][4];
@@ -499,7 +499,12 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
         __syncwarp();
         tc_fence_before();
     }
-    if (!ok && lane == 0 && g.status) g.status[box] = HPS_ETIMEOUT;
+    if (lost >= 0) {
+        if (lane == 0 && g.status) g.status[box] = HPS_ETIMEOUT;
+        // no tile is issued any more; the one that was lost and the next, already issued, end before TMEM is freed
+        if (warp == 0)
+            for (int t = lost; t < min(lost + 2, cnt); ++t) wait(&tfull[t & 1], t >> 1);
+    }
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
