@@ -198,14 +198,13 @@ void lu_factor(const Plan& P, Work<T>& w, int nbox, int* status, cudaStream_t st
 {
     const int n = P.n, NB = P.NB;
     const long long ldm = P.ldm;
-    if constexpr (sizeof(T) == 8) launch_wide(w.M, ldm, w.sM, n, P.axis, P.dims, w.wide, nbox, st);
     for (int s = 0; s < P.nsteps; ++s) {
         const int k = P.k0[s], nb = P.nbs[s];
         T* Fs = w.F + P.fw_off[s];
         T* Bs = w.B + P.bw_off[s];
         int* Ps = w.perm + P.perm_off[s];
         launch_panel<T>(w.M, ldm, w.sM, n, k, nb, Ps, w.sP, Fs, NB, w.sF, Bs + (long long)k * NB, NB, w.sB,
-                        status, nullptr, w.wide, nbox, st);
+                        status, nullptr, w.wide, P.axis, P.dims, nbox, st);
         if (n - k - nb > 0) {
             GemmArgs<T> a = gargs<T>(w);
             a.A = w.M + (long long)(k + nb) * ldm + k; a.lda = ldm; a.sA = w.sM;

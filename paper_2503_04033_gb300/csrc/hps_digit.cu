@@ -21,7 +21,7 @@
 //
 // So the only roundings are those three; a plain FP64 sum rounds K times, but
 // relative to its own terms, not to the scales: operands whose scales say little
-// about an entry are summed plainly on the FP64 pipe (CHECK below, launch_wide).
+// about an entry are summed plainly on the FP64 pipe (CHECK below; is_wide in hps_panel.cu).
 // Against a higher-precision solve, the LU built on these products is as close
 // as or closer than the one on FP64 multiply-adds (tests/test_gpu_digit.py).
 // Results outside the normal range, and all of a row or column that holds an
@@ -240,7 +240,7 @@ __device__ __noinline__ void plain_tiles(const DgArgs& a)
 // meets another one (a bit per factor, joined by AND), or where nothing but zeros
 // meet.  Every other entry, and those of rows and columns with subnormals, are
 // summed as they stand on the FP64 pipe.  LU products go by their matrix instead
-// (see launch_wide).
+// (is_wide, hps_panel.cu).
 template <bool BT, bool CHECK>
 __global__ void __launch_bounds__(DG_THREADS, 1)
 k_digit_gemm(const __grid_constant__ DgArgs a)
@@ -257,11 +257,8 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
     if (g.skip && g.skip[box]) return;
     const int t0 = blockIdx.x * a.per, cnt = min(a.per, a.tiles_n - t0);
     if (cnt <= 0) return;
-    if constexpr (!CHECK)
-        if (g.wide[box]) {
-            plain_tiles(a);
-            return;
-        }
+    int hard = 0;   // read here, needed once the operands' loads are on their way
+    if constexpr (!CHECK) hard = g.wide[box];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = blockIdx.y * DG_BM;
     const uint32_t sb = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -276,7 +273,6 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
         mbar_init(smem_u32(&tfull[1]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), 512);
     if (tid < 4 * DG_BN) (&colE[0][0])[tid] = E_MIN;
     if (tid < DG_BM) {
         const int r = m0 + tid;
@@ -321,6 +317,12 @@ k_digit_gemm(const __grid_constant__ DgArgs a)
             for (int u = 0; u < 4; ++u) x[ps][u] = (r < g.M && k + u < g.K) ? A[(long long)r * g.lda + k + u] : 0.0;
         }
         load_b(t0);
+        if constexpr (!CHECK)
+            if (hard) {   // the whole box
+                plain_tiles(a);
+                return;
+            }
+        if (warp == 0) tmem_alloc(smem_u32(&tmem_sh), 512);
 #pragma unroll
         for (int ps = 0; ps < 4; ++ps) {
             const int rl = ps * 32 + (tid >> 4);

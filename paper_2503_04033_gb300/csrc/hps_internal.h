@@ -129,21 +129,6 @@ struct GemmArgs {
     const int* wide;                 // FP64: per box, nonzero = plain FP64 sums (NULL: the product looks at each entry)
 };
 
-// FP64 LUs run from exact digits (hps_digit.cu), which are as good as FP64 sums
-// relative to the largest entries of a row and a column of a product.  A matrix
-// whose scales lie far apart needs its small entries too, and its LU runs on
-// plain sums: launch_wide sets wide[box] where the rows' largest entries lie 2^9
-// or more apart, or (axis, dims: a collocation matrix of axis^dims nodes) where
-// the second differences of its axes do by more than 2^12.  Measured on S
-// against long double, digits : FP64 sums (geometric means of the norms of the
-// errors): rows 2^7 apart, as in every smooth, rough or cross-term problem here
-// (p <= 24), 0.5 to 1; 2^10 (impedance leaves of side 1 / 64) 5; 2^13
-// (coefficients that jump by 1e8 from node to node) 1.4, 19 at worst; 2^27 20,
-// 5e4 at worst.  Sides 1 : 10 and 1 : 100 0.7, but 8 and 16 for the median entry
-// of S, and 1 : 1e6 all but three digits of the small ones.
-void launch_wide(const double* M, long long ldm, long long sM, int n, int axis, int dims, int* wide, int nbox,
-                 cudaStream_t st);
-
 // ---------------------------------------------------------------- LU plans
 
 struct Plan {
@@ -247,7 +232,7 @@ struct Work {
     float *it1, *it2;   // format 2: 1 / (power-of-two scale) of each column of the G in Gp, Gp2
     double* norms;
     int* skip;
-    int* wide;     // FP64: boxes that run on plain sums
+    int* wide;     // FP64: boxes that run on plain sums (judged by the LU's first panel, hps_panel.cu)
     long long sM, sF, sB, sG, sP, sX, sFp, sBp, sGp, sRC, sIT;
 };
 
@@ -319,7 +304,7 @@ void launch_build_aug(const Geometry& g, double kappa, const double* kappa_box, 
 template <typename T>
 void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* perm, long long sP, T* Ftop,
                   long long ldf, long long sF, T* Btop, long long ldb, long long sB, int* status, const int* skip,
-                  const int* wide, int nbox, cudaStream_t st);
+                  int* wide, int axis, int dims, int nbox, cudaStream_t st);
 
 template <typename T>
 void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c0, int ncols,

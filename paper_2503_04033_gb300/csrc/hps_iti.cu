@@ -53,7 +53,7 @@ __global__ void k_iti_tables(const ItiTables a, double* D, double* D2)
 // [3][p][p] (axis-major), b [nbox][p^3].  The face rows of axis a, of order
 // 1 / h_a, are written times scale[a], the power of two that brings them to the
 // interior rows' order 1 / h^2: the LU's products share a scale per row and
-// column (see launch_wide), and with the rows as they come R was 5 (side 1 / 64) to
+// column (is_wide, hps_panel.cu), and with the rows as they come R was 5 (side 1 / 64) to
 // 1000 times (1 / 1024) further from long double than on FP64 sums.
 __global__ void __launch_bounds__(256)
 k_build_iti(int p, int n, int m, const double* __restrict__ D, const double* __restrict__ D2, double kappa2,

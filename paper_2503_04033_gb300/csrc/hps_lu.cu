@@ -1267,50 +1267,6 @@ void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c
     prof_end(KC_GATHER, st, 0.0, (double)nbox * nb * (double)ncols * sizeof(T) * (W ? 3 : 2));
 }
 
-// See launch_wide.  A row's scale is the exponent of its largest entry within two
-// columns of the diagonal, where collocation, impedance and interface matrices
-// have entries of that size (all of M would take 0.7 ms to read of the 101 of 512
-// boxes at p = 12).  The axes are compared along the grid's diagonal, where the
-// neighbours on every axis have the same 1-D index; half of these nodes decide.
-__global__ void k_wide(const double* __restrict__ M, long long ldm, long long sM, int n, int axis, int dims, int* wide)
-{
-    __shared__ int top[2], flat;   // largest exponent, 2047 less the smallest; nodes with axes far apart
-    if (threadIdx.x == 0) top[0] = top[1] = flat = 0;
-    __syncthreads();
-    const double* A = M + blockIdx.x * sM;
-    auto expo = [&](long long r, long long c) { return ((unsigned)__double2hiint(A[r * ldm + c]) & 0x7FFFFFFFu) >> 20; };
-    int hi = 0, lo = 0;
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
-        unsigned e[5];
-#pragma unroll
-        for (int u = 0; u < 5; ++u) e[u] = expo(r, min(max(r + u - 2, 0), n - 1));
-        const int t = (int)max(max(max(e[0], e[1]), max(e[2], e[3])), e[4]);
-        hi = max(hi, t);
-        lo = max(lo, 2047 - t);
-    }
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    lo = __reduce_max_sync(0xffffffffu, lo);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&top[0], hi);
-        atomicMax(&top[1], lo);
-    }
-    if (dims && (int)threadIdx.x + 1 < axis) {
-        const long long node = 1 + axis + (dims == 3 ? (long long)axis * axis : 0), r = threadIdx.x * node;
-        const unsigned x = expo(r, r + 1), y = expo(r, r + axis), z = dims == 3 ? expo(r, r + (long long)axis * axis) : x;
-        if (max(max(x, y), z) > min(min(x, y), z) + 12) atomicAdd(&flat, 1);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) wide[blockIdx.x] = top[0] + top[1] >= 2047 + 9 || (dims && 2 * flat >= axis - 1 && flat > 0);
-}
-
-void launch_wide(const double* M, long long ldm, long long sM, int n, int axis, int dims, int* wide, int nbox,
-                 cudaStream_t st)
-{
-    prof_begin(KC_MISC, st);
-    k_wide<<<(unsigned)nbox, 256, 0, st>>>(M, ldm, sM, n, axis, dims, wide);
-    prof_end(KC_MISC, st, 0.0, (double)nbox * n * 5 * 8.0);
-}
-
 // FP64 products run from exact digits on the tensor cores at every size, the
 // smallest included: 4096 boxes at p = 3 (products of 1 x 6 x 1) take 1000 us a
 // call against 1390 on the FP64 pipes, p = 4 (8 x 24 x 8) 1267 : 1677, p = 5

@@ -261,8 +261,59 @@ struct PanelArgs {
     long long sP;
     int* status;
     const int* skip;
-    const int* wide;   // FP64: boxes whose left products run as plain sums (see launch_wide)
+    int* wide;       // FP64: boxes that run on plain sums (is_wide; written by the panel at k = 0)
+    int axis, dims;
 };
+
+// FP64 LUs run from exact digits (hps_digit.cu), which are as good as FP64 sums
+// relative to the largest entries of a row and a column of a product.  A matrix
+// whose scales lie far apart needs its small entries too, and its LU runs on
+// plain sums: true where the rows' largest entries lie 2^9 or more apart, or (axis,
+// dims: a collocation matrix of axis^dims nodes) where the second differences of
+// its axes do by more than 2^12.  Measured on S against long double, digits : FP64
+// sums (geometric means of the norms of the errors): rows 2^7 apart, as in every
+// smooth, rough or cross-term problem here (p <= 24), 0.5 to 1; 2^10 (impedance
+// leaves of side 1 / 64 before their rows were scaled) 5; 2^13 (coefficients that
+// jump by 1e8 from node to node) 1.4, 19 at worst; 2^27 20, 5e4 at worst.  Sides
+// 1 : 10 and 1 : 100 0.7, but 8 and 16 for the median entry of S, and 1 : 1e6 all
+// but three digits of the small ones.
+//
+// A row's scale is the exponent of its largest entry within two columns of the
+// diagonal, where collocation, impedance and interface matrices have entries of
+// that size (all of M would take 0.7 ms to read of the 101 of 512 boxes at p =
+// 12).  The axes are compared along the grid's diagonal, where the neighbours on
+// every axis have the same 1-D index; half of these nodes decide.  Every CTA of the
+// first panel finds the same answer for itself: a kernel for it took 5 of the 117
+// us of one box at p = 5.
+__device__ __noinline__ bool is_wide(const double* __restrict__ A, long long ldm, int n, int axis, int dims)
+{
+    __shared__ int top[2], flat;   // largest exponent, 2047 less the smallest; nodes with axes far apart
+    if (threadIdx.x == 0) top[0] = top[1] = flat = 0;
+    __syncthreads();
+    auto expo = [&](long long r, long long c) { return ((unsigned)__double2hiint(A[r * ldm + c]) & 0x7FFFFFFFu) >> 20; };
+    int hi = 0, lo = 0;
+    for (int r = threadIdx.x; r < n; r += PT) {
+        unsigned e[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) e[u] = expo(r, min(max(r + u - 2, 0), n - 1));
+        const int t = (int)max(max(max(e[0], e[1]), max(e[2], e[3])), e[4]);
+        hi = max(hi, t);
+        lo = max(lo, 2047 - t);
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&top[0], hi);
+        atomicMax(&top[1], lo);
+    }
+    if (dims && (int)threadIdx.x + 1 < axis) {
+        const long long node = 1 + axis + (dims == 3 ? (long long)axis * axis : 0), r = threadIdx.x * node;
+        const unsigned x = expo(r, r + 1), y = expo(r, r + axis), z = dims == 3 ? expo(r, r + (long long)axis * axis) : x;
+        if (max(max(x, y), z) > min(min(x, y), z) + 12) atomicAdd(&flat, 1);
+    }
+    __syncthreads();
+    return top[0] + top[1] >= 2047 + 9 || (dims && 2 * flat >= axis - 1 && flat > 0);
+}
 
 // Entry (row, column) of the product of an earlier block's multipliers with u as
 // an FP64 sum; l, u: the first multiplier and value, a step apart each.
@@ -320,7 +371,7 @@ k_panel(const PanelArgs<T> a)
     const int R0 = a.n - a.k;
     T* P = a.M + box * a.sM + (long long)a.k * a.ldm + a.k;   // the panel's corner
     bool hard = false;   // FP64: left products as plain sums
-    if constexpr (sizeof(T) == 8) hard = a.wide[box] != 0;
+    if constexpr (sizeof(T) == 8) hard = a.k == 0 ? is_wide(P, a.ldm, a.n, a.axis, a.dims) : a.wide[box] != 0;
     auto row_of = [&](int rr) { return ((rr * PW + warp) * C + rank) * 32 + lane; };
     // the warp's row groups that exist (all of a group's lanes may still be past the last row)
     const int nrr = min(RPT, max(0, ((R0 + 31) / 32 - rank - warp * C + PW * C - 1) / (PW * C)));
@@ -443,7 +494,7 @@ k_panel(const PanelArgs<T> a)
                 // (K = IB <= 16: every accumulator stays below 2^21); as 16 multiply-adds
                 // per entry on the FP64 pipe, 64 clocks a warp each, it took seven times as long
                 const int g = lane >> 2, q = lane & 3;
-                if (warp < IB / 8 && !hard) {
+                if (warp < IB / 8) {
                     double v[4];
                     int ex = E_MIN;
 #pragma unroll
@@ -461,20 +512,6 @@ k_panel(const PanelArgs<T> a)
                     if (q == 0) s.ue[8 * warp + g] = ex == E_BAD ? E_NAN : ex - 1018;
                 }
                 __syncthreads();
-                if (hard) {
-#pragma unroll 1
-                    for (int kk = 0; kk < IB; ++kk)
-#pragma unroll
-                        for (int rr = 0; rr < RPT; ++rr) {
-                            const bool on = pidx[rr] == -1 || pidx[rr] >= je + IB;
-                            const T l = on ? Lt[(long long)(je + kk) * R0 + row_of(rr)] : T(0);
-                            if (on) {
-#pragma unroll
-                                for (int c = 0; c < IB; ++c) x[rr][c] -= l * s.u[kk][c];
-                            }
-                        }
-                    continue;
-                }
 #pragma unroll
                 for (int rr = 0; rr < RPT; ++rr) {
                     if (rr >= nrr) continue;
@@ -500,7 +537,7 @@ k_panel(const PanelArgs<T> a)
                             ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 1));
                             ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 2));
                             split4(v, ex, ad[h]);
-                            ea[h] = ex == E_BAD ? E_NAN : ex;
+                            ea[h] = ex == E_BAD || hard ? E_NAN : ex;   // E_NAN: every entry of the row a plain sum
                         }
 #pragma unroll 1
                         for (int nt = 0; nt < IB / 8; ++nt) {
@@ -743,6 +780,8 @@ k_panel(const PanelArgs<T> a)
         }
     }
     if (rank != 0) return;
+    if constexpr (sizeof(T) == 8)
+        if (tid == 0 && a.k == 0) a.wide[box] = hard;
 
     // The pivot rows on top: their multipliers of earlier blocks join what LU holds.
     for (int idx = tid; idx < nb * ldl; idx += PT) {
@@ -952,7 +991,7 @@ __global__ void k_refuse(int nbox, int* status)
 template <typename T>
 void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* perm, long long sP, T* Ftop,
                   long long ldf, long long sF, T* Btop, long long ldb, long long sB, int* status, const int* skip,
-                  const int* wide, int nbox, cudaStream_t st)
+                  int* wide, int axis, int dims, int nbox, cudaStream_t st)
 {
     panel_attributes<T>();
     // Rows per thread and cluster size: the fewest waves of (chain of a pivot +
@@ -991,7 +1030,7 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
     // multiple of 8 and k one of 16 (make_plan rounds every stride up, steps are
     // NB wide).  The multipliers' scratch is the step's F block, which the inverse and the
     // product after this overwrite
-    PanelArgs<T> a{M, ldm, sM, n, k, nb, Ftop, sF, perm, sP, status, skip, wide};
+    PanelArgs<T> a{M, ldm, sM, n, k, nb, Ftop, sF, perm, sP, status, skip, wide, axis, dims};
     prof_begin(KC_PANEL, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nbox * bc));
@@ -1014,8 +1053,8 @@ void launch_panel(T* M, long long ldm, long long sM, int n, int k, int nb, int* 
 }
 
 template void launch_panel<float>(float*, long long, long long, int, int, int, int*, long long, float*, long long,
-                                  long long, float*, long long, long long, int*, const int*, const int*, int, cudaStream_t);
+                                  long long, float*, long long, long long, int*, const int*, int*, int, int, int, cudaStream_t);
 template void launch_panel<double>(double*, long long, long long, int, int, int, int*, long long, double*, long long,
-                                   long long, double*, long long, long long, int*, const int*, const int*, int, cudaStream_t);
+                                   long long, double*, long long, long long, int*, const int*, int*, int, int, int, cudaStream_t);
 
 }  // namespace hps

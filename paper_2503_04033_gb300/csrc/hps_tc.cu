@@ -1675,7 +1675,7 @@ bool tc_lu_factor(const Plan& P, Work<float>& w, int nbox, int* status, cudaStre
         float* Bs = w.B + P.bw_off[s];
         int* Ps = w.perm + P.perm_off[s];
         launch_panel<float>(w.M, ldm, w.sM, n, k, nb, Ps, w.sP, Fs, NB, w.sF, Bs + (long long)k * NB, NB,
-                            w.sB, status, nullptr, nullptr, nbox, st);
+                            w.sB, status, nullptr, nullptr, 0, 0, nbox, st);
         // F rows below the panel, L21 L11^{-1} = -(L21 * F_top), and B rows above
         // it, U01 U11^{-1} = -(U01 * B_top), as tensor-core products: the left
         // operand is split into the step's own (not yet filled) pack region,
