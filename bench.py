@@ -70,10 +70,10 @@ def operand_format(prec, opts):
     if float(opts.get("FP16_OPERANDS", 1)) != 0:
         return "scaled 2 x FP16", 1.0, 3
     return "3 x TF32", TF32_OVER_BF16, 3
-# FP64 issue rate: 152 SMs x 2070 MHz x 2 FP64 FMA/clk/SM x 2 flop (1.26
-# TFLOP/s, the part's nominal 1.25 TFLOP/s); used only where a run has not
-# measured its own FP64 matmul rate.
-FP64_PEAK_TFLOPS = 152 * 2.070e9 * 2 * 2 / 1e12
+
+# FP16 digit pairs behind a multiply-add of the FP64 products (hps_digit.cu):
+# the bound of FP64 work is the dense FP16 rate over this.
+FP64_DIGIT_PAIRS = 36
 # DRAM bytes per launch of the tensor-core update products at 512 boxes, by
 # operand format: dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture of the factorisation phase at 32 boxes, per launch, times 16 (the
@@ -166,7 +166,7 @@ def measured_peaks():
 def measured_matmul_peaks(dev):
     """Dense matmul rates measured here with torch (cuBLAS): FP64 at 4096^3
     and FP16 / BF16 at 8192^3, best of 5 after a warm-up, CUDA events.  The
-    FP64 figure is the peak of the plain FP64 GPU path and the FP64 kernels;
+    FP64 figure is cuBLAS's rate on the FP64 pipes;
     the FP16 one checks that FP16 runs at the BF16 rate."""
     import torch
     out = {}
@@ -188,6 +188,15 @@ def measured_matmul_peaks(dev):
     torch.cuda.empty_cache()
     out["how"] = "torch.matmul best of several, CUDA events; FP64 4096^3, FP16/BF16 8192^3 (burst)"
     return out
+
+
+def _digit_roofline(tflops):
+    """Roofline of a whole FP64 leaf call against the rate at which the tensor cores can do its products."""
+    peaks, src = measured_peaks()
+    peak = peaks["bf16_tflops_sustained"] / FP64_DIGIT_PAIRS
+    return {"bound": "tensor", "achieved": tflops, "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
+            "traffic": None, "peak_source": f"{src} sustained BF16 dense peak / {FP64_DIGIT_PAIRS} digit pairs a "
+                                            "multiply-add (FP16 has the same rate); the whole call"}
 
 
 class ClockSampler:
@@ -416,7 +425,8 @@ def run_ours(args):
     line["measured_matmul_peaks"] = mm
     fmt_name, rate, nmma = operand_format(prec, opts)
     if prec == H.HPS_FP64:
-        tpeak, tsrc = mm["fp64_tflops"], "torch float64 matmul measured in this run (4096^3)"
+        tpeak = peaks["bf16_tflops_sustained"] / FP64_DIGIT_PAIRS
+        tsrc = f"{src} sustained BF16 dense peak / {FP64_DIGIT_PAIRS} digit pairs a multiply-add"
     else:
         tpeak = peaks["bf16_tflops_sustained"] * rate
         tsrc = (f"{src} sustained BF16 dense peak" + (" (FP16 has the same nominal rate)" if rate == 1.0 else
@@ -1271,10 +1281,7 @@ def run_leaf2d(args):
                                    "b = 1 + 0.4 sin(6x) cos(4y), one load f = cos(3x + y)",
                        "l2": "inputs and workspace larger than L2, no flush"},
             "tflops": tflops,
-            "roofline": {"bound": "alu", "achieved": tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": tflops / FP64_PEAK_TFLOPS, "traffic": None,
-                         "peak_source": "FP64 issue rate 152 SMs x 2.07 GHz x 2 FMA/clk (the whole call; its LU products "
-                                        "run from exact digits on the tensor cores, so frac can pass 1)"},
+            "roofline": _digit_roofline(tflops),
             "rel_err_vs_oracle_max": worst, "box_failures": fails, "clocks": clocks.summary(),
             "cpu_baseline": {"value": len(sel) / cpu_s, "unit": "boxes/s", "cores": oracle.max_threads(),
                              "kind": "oracle", "sample": f"{len(sel)} boxes spread over the grid, 2-D FP64 oracle "
@@ -1291,10 +1298,7 @@ def _fp64_leaf_line(metric, value, ms, args, workload, flops_per_box, worst, fai
             "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": workload, "l2": "inputs and workspace larger than L2, no flush"},
             "tflops": tflops,
-            "roofline": {"bound": "alu", "achieved": tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": tflops / FP64_PEAK_TFLOPS, "traffic": None,
-                         "peak_source": "FP64 issue rate 152 SMs x 2.07 GHz x 2 FMA/clk (the whole call; its LU products "
-                                        "run from exact digits on the tensor cores, so frac can pass 1)"},
+            "roofline": _digit_roofline(tflops),
             "rel_err_vs_oracle_max": worst, "box_failures": fails, "clocks": clocks.summary(),
             "cpu_baseline": {"value": cpu_rate, "unit": "boxes/s", "cores": oracle.max_threads(), "kind": "oracle",
                              "sample": f"{cpu_n} boxes spread over the batch, FP64 oracle, one box at a time"}}

@@ -270,13 +270,13 @@ struct PanelArgs {
 // whose scales lie far apart needs its small entries too, and its LU runs on
 // plain sums: true where the rows' largest entries lie 2^9 or more apart, or (axis,
 // dims: a collocation matrix of axis^dims nodes) where the second differences of
-// its axes do by more than 2^12.  Measured on S against long double, digits : FP64
-// sums (geometric means of the norms of the errors): rows 2^7 apart, as in every
-// smooth, rough or cross-term problem here (p <= 24), 0.5 to 1; 2^10 (impedance
-// leaves of side 1 / 64 before their rows were scaled) 5; 2^13 (coefficients that
-// jump by 1e8 from node to node) 1.4, 19 at worst; 2^27 20, 5e4 at worst.  Sides
-// 1 : 10 and 1 : 100 0.7, but 8 and 16 for the median entry of S, and 1 : 1e6 all
-// but three digits of the small ones.
+// its axes do by more than 2^12.  Errors of S against long double, from digits :
+// on FP64 sums (geometric means of norms over ten 2-D boxes, p = 16): rows 2^5
+// apart (every smooth or rough problem; at most 2^7 at p <= 24) 1 : 1.3, 2^13
+// (coefficients that jump by 1e8 from node to node) 1.2 : 1, 2^19 to 2^33 (1e10 to
+// 1e14) 19 to 26 : 1, 2^39 (1e16) 1500 : 1; impedance leaves of side 1 / 64, 2^10
+// apart before their rows were scaled, 15 : 1.  Boxes of sides 1 : 100 keep the norm
+// but lose a digit of the median entry, 1 : 1e6 all but two of the small ones.
 //
 // A row's scale is the exponent of its largest entry within two columns of the
 // diagonal, where collocation, impedance and interface matrices have entries of
