@@ -281,7 +281,8 @@ struct PanelArgs {
 // A row's scale is the exponent of its largest entry within two columns of the
 // diagonal, where collocation, impedance and interface matrices have entries of
 // that size (all of M would take 0.7 ms to read of the 101 of 512 boxes at p =
-// 12).  The axes are compared along the grid's diagonal, where the neighbours on
+// 12); rows with nothing beside it, the identity that pads a separator to its
+// level's size, have none.  The axes are compared along the grid's diagonal, where the neighbours on
 // every axis have the same 1-D index; half of these nodes decide.  Every CTA of the
 // first panel finds the same answer for itself: a kernel for it took 5 of the 117
 // us of one box at p = 5.
@@ -293,12 +294,15 @@ __device__ __noinline__ bool is_wide(const double* __restrict__ A, long long ldm
     auto expo = [&](long long r, long long c) { return ((unsigned)__double2hiint(A[r * ldm + c]) & 0x7FFFFFFFu) >> 20; };
     int hi = 0, lo = 0;
     for (int r = threadIdx.x; r < n; r += PT) {
-        unsigned e[5];
+        unsigned beside = 0;
 #pragma unroll
-        for (int u = 0; u < 5; ++u) e[u] = expo(r, min(max(r + u - 2, 0), n - 1));
-        const int t = (int)max(max(max(e[0], e[1]), max(e[2], e[3])), e[4]);
-        hi = max(hi, t);
-        lo = max(lo, 2047 - t);
+        for (int u = -2; u <= 2; ++u)
+            if (u != 0 && r + u >= 0 && r + u < n) beside = max(beside, expo(r, r + u));
+        const int t = (int)max(beside, expo(r, r));
+        if (beside) {
+            hi = max(hi, t);
+            lo = max(lo, 2047 - t);
+        }
     }
     hi = __reduce_max_sync(0xffffffffu, hi);
     lo = __reduce_max_sync(0xffffffffu, lo);
