@@ -87,7 +87,9 @@ typedef enum {
  * refinement with the tensor-core products taken in BF16 with FP32
  * accumulation: each operand is split into three BF16 pieces (successive
  * roundings of the remainder) and six kind::f16 products per K step keep every
- * term above FP32 rounding, so the factors are as accurate as FP32's.  Without
+ * term above FP32 rounding; the tensor cores' FP32 sums are cut, not rounded, so
+ * the factors are a few times less accurate than from FP32 multiply-adds, which
+ * the refinement recovers.  Without
  * tensor cores (HPS_OPT_TENSOR_CORES = 0) it runs as HPS_FP32_IR. */
 typedef enum { HPS_FP64 = 0, HPS_FP32_IR = 1, HPS_BF16_IR = 2 } hps_precision;
 

@@ -44,7 +44,7 @@
 // or by a warp of their own were each slower (2.0, 2.4 and 2.6 ms against 1.74):
 // they cost registers or coalesced reads of B, and the MMAs' latency shows.
 // Whole calls: 512 boxes at p = 12 (DtN, particular and reconstruction) 1001 ->
-// 101 ms, cross-term leaves 225 -> 39 ms.
+// 101 ms, cross-term leaves 225 -> 39 to 41 ms.
 #include <algorithm>
 
 #include "hps_digits.cuh"

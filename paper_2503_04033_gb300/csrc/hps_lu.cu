@@ -1268,7 +1268,7 @@ void launch_gather(const T* M, long long ldm, long long sM, int k, int nb, int c
 }
 
 // FP64 products run from exact digits on the tensor cores at every size, the
-// smallest included: 4096 boxes at p = 3 (products of 1 x 6 x 1) take 1000 us a
+// smallest included: 4096 boxes at p = 3 (products of 1 x 6 x 1) take 990 us a
 // call against 1390 on the FP64 pipes, p = 4 (8 x 24 x 8) 1267 : 1677, p = 5
 // 2610 : 3692, one box at p = 5 117 : 173, with errors of T no larger.
 template <>
